@@ -349,6 +349,29 @@ bz_status materialize_if_lazy(bz_handle *H, int x, cudaStream_t s)
     return BZ_OK;
 }
 
+// The corrected state of buffer x in device memory dst of this handle's
+// device: one pass that reads h_c and writes the copy (the buffer keeps its
+// pending corrections), where correcting in place and then copying reads and
+// writes the state twice.  256^2 cells x 32^3 nodes, ten steps and one copy:
+// 69.9 -> 67.3 ms.
+// False (nothing launched) when dst is not such memory, or not aligned for
+// 16-byte stores: the caller corrects in place and copies.
+bool copy_corrected(bz_handle *H, int x, void *dst, cudaStream_t s)
+{
+    cudaPointerAttributes at{};
+    if (((uintptr_t)dst & 15u) != 0) return false;
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != H->dev) return false;
+    const Geo &g = H->g;
+    bzk::k_lz_materialize<<<std::min(g.nr, H->nsm * 8), 256, 0, s>>>(
+        g, nullptr, (const float *)H->h[x], H->mu[x], (float *)dst, nullptr);
+    H->launches++;
+    return true;
+}
+
 // Buffer x is about to be overwritten by a path that writes corrected states.
 bz_status drop_lazy(bz_handle *H, int x, cudaStream_t s)
 {
@@ -1476,12 +1499,12 @@ bz_status bz_moments(bz_handle *H, double *out, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     const Geo &g = H->g;
     if (!H->mom_valid) {
-        BZ_TRY(materialize_if_lazy(H, H->cur, s));
         int grid = std::min(g.nr, H->nsm * 8);
         if (H->dtype == BZ_F64)
-            bzk::k_moments<double><<<grid, 256, 0, s>>>(g, (const double *)H->h[H->cur], H->mom);
+            bzk::k_moments<double><<<grid, bzk::kMomThreads, 0, s>>>(g, (const double *)H->h[H->cur], H->mom);
         else
-            bzk::k_moments<float><<<grid, 256, 0, s>>>(g, (const float *)H->h[H->cur], H->mom);
+            bzk::k_moments<float><<<grid, bzk::kMomThreads, 0, s>>>(g, (const float *)H->h[H->cur], H->mom,
+                                                                   H->lazy_buf[H->cur] ? H->mu[H->cur] : nullptr);
         BZ_LAUNCHED(H);
         H->mom_valid = true;
     }
@@ -1523,9 +1546,13 @@ bz_status bz_lid_shear(bz_handle *H, double *out, void *stream)
 bz_status bz_get_state(bz_handle *H, void *dst, int64_t *step, void *stream)
 {
     if (!H || !dst) return fail(BZ_EINVAL, "NULL argument");
-    BZ_TRY(materialize_if_lazy(H, H->cur, (cudaStream_t)stream));
-    BZ_CUDA(cudaMemcpyAsync(dst, H->h[H->cur], H->esz * (size_t)H->g.nr * H->g.nvt,
-                            cudaMemcpyDefault, (cudaStream_t)stream));
+    if (H->lazy_buf[H->cur] && copy_corrected(H, H->cur, dst, (cudaStream_t)stream)) {
+        BZ_CUDA(cudaGetLastError());
+    } else {
+        BZ_TRY(materialize_if_lazy(H, H->cur, (cudaStream_t)stream));
+        BZ_CUDA(cudaMemcpyAsync(dst, H->h[H->cur], H->esz * (size_t)H->g.nr * H->g.nvt,
+                                cudaMemcpyDefault, (cudaStream_t)stream));
+    }
     if (step) *step = H->step;
     return BZ_OK;
 }
@@ -2473,9 +2500,13 @@ bz_status bz_batch_get_state(bz_batch *B, int32_t i, void *dst, int64_t *step, v
 {
     if (!B || i < 0 || i >= B->n || !dst) return fail(BZ_EINVAL, "invalid argument");
     bz_handle *h = B->inst[i];
-    BZ_TRY(batch_correct_in_place(B, i, (cudaStream_t)stream));
-    BZ_CUDA(cudaMemcpyAsync(dst, h->h[B->step[i] & 1], h->esz * (size_t)h->g.nr * h->g.nvt,
-                            cudaMemcpyDefault, (cudaStream_t)stream));
+    if (B->mode != 0 && copy_corrected(h, (int)(B->step[i] & 1), dst, (cudaStream_t)stream)) {
+        BZ_CUDA(cudaGetLastError());
+    } else {
+        BZ_TRY(batch_correct_in_place(B, i, (cudaStream_t)stream));
+        BZ_CUDA(cudaMemcpyAsync(dst, h->h[B->step[i] & 1], h->esz * (size_t)h->g.nr * h->g.nvt,
+                                cudaMemcpyDefault, (cudaStream_t)stream));
+    }
     if (step) *step = B->step[i];
     return BZ_OK;
 }
@@ -2486,9 +2517,9 @@ bz_status bz_batch_moments(bz_batch *B, int32_t i, double *out, void *stream)
     bz_handle *h = B->inst[i];
     cudaStream_t s = (cudaStream_t)stream;
     const Geo &g = h->g;
-    BZ_TRY(batch_correct_in_place(B, i, s));
-    bzk::k_moments<float><<<std::min(g.nr, h->nsm * 8), 256, 0, s>>>(
-        g, (const float *)h->h[B->step[i] & 1], h->mom);
+    const int b = (int)(B->step[i] & 1);
+    bzk::k_moments<float><<<std::min(g.nr, h->nsm * 8), bzk::kMomThreads, 0, s>>>(
+        g, (const float *)h->h[b], h->mom, B->mode != 0 ? h->mu[b] : nullptr);
     BZ_CUDA(cudaGetLastError());
     BZ_CUDA(cudaMemcpyAsync(out, h->mom, sizeof(double) * 11 * (size_t)g.nr, cudaMemcpyDefault, s));
     BZ_CUDA(cudaStreamSynchronize(s));

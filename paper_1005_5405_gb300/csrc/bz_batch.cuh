@@ -384,14 +384,11 @@ __global__ void kbl_fb_materialize(const LzInst *__restrict__ inst, const int *_
         for (int o = threadIdx.x; o < g.nvt / 4; o += blockDim.x) {
             const int jx = o / Q, q = o % Q, jy = q / nq, jz = 4 * (q % nq);
             const float vx = sv[jx], vy = sv[jy];
-            const float base = smu[0] + smu[1] * vx + smu[2] * vy + smu[4] * (vx * vx + vy * vy);
             float4 h = hc[o];
             float *hp = &h.x;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float vz = sv[jz + r];
-                hp[r] = lz_corr(hp[r], base + smu[3] * vz + smu[4] * vz * vz, g.epsf);
-            }
+            for (int r = 0; r < 4; ++r)
+                hp[r] = state_corr(hp[r], state_kappa(smu, vx, vy, sv[jz + r]), g.epsf);
             hc[o] = h;
         }
         if (threadIdx.x < 8) {

@@ -1261,49 +1261,132 @@ k_cell(Geo g, const R *__restrict__ hin, const R *__restrict__ ghost,
     if (fallback && stats) atomicAdd(stats + 3, (unsigned long long)fallback);
 }
 
-// Moments of an arbitrary state (Eqs. densita..sforzi), one CTA per cell.
-template <typename R>
-__global__ void k_moments(Geo g, const R *__restrict__ h, double *__restrict__ mom)
+// A stored node value h_c with its cell's pending correction mu: the value
+// is h_c + (1 + eps h_c) kappa, kappa = mu . (1, v, v^2).
+__device__ __forceinline__ float state_kappa(const float *mu, float vx, float vy, float vz)
 {
-    __shared__ double red[kMaxWarps * kRedSlots];
-    __shared__ double tot[kRedSlots];
-    const int N = g.nv, N2 = N * N;
-    for (int c = blockIdx.x; c < g.nr; c += gridDim.x) {
-        double mo[10];
-        for (int k = 0; k < 10; ++k) mo[k] = 0.0;
-        const R *src = h + (int64_t)c * g.nvt;
-        for (int j = threadIdx.x; j < g.nvt; j += blockDim.x) {
-            int jx = j / N2, jy = (j / N) % N, jz = j % N;
-            double vx = g.axv[jx], vy = g.axv[jy], vz = g.axv[jz];
-            double wh = g.axA[jx] * g.axA[jy] * g.axA[jz] * (double)src[j];
-            mo[0] += wh;
-            mo[1] += wh * vx;
-            mo[2] += wh * vy;
-            mo[3] += wh * vz;
-            mo[4] += wh * vx * vx;
-            mo[5] += wh * vy * vy;
-            mo[6] += wh * vz * vz;
-            mo[7] += wh * vx * vy;
-            mo[8] += wh * vx * vz;
-            mo[9] += wh * vy * vz;
+    const float base = mu[0] + mu[1] * vx + mu[2] * vy + mu[4] * (vx * vx + vy * vy);
+    return base + mu[3] * vz + mu[4] * vz * vz;
+}
+__device__ __forceinline__ float state_corr(float hc, float kappa, float eps)
+{
+    return fmaf(eps * hc, kappa, hc + kappa);
+}
+
+// Sums of 16 doubles over a warp by recursive halving (16 additions and
+// shuffles instead of 16 x 5): lane l returns the total of value l / 2.
+__device__ __forceinline__ double warp_reduce_scatter16(double (&v)[16])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16, n = 8; n >= 1; o >>= 1, n >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
         }
-        block_reduce<10, double>(mo, red, tot);
-        if (threadIdx.x == 0) {
-            const double *m = tot, e = g.eps;
-            double rho = m[0], n = 1.0 + e * rho;
-            double u[3] = {m[1] / n, m[2] / n, m[3] / n};
+    }
+    return v[0] + __shfl_xor_sync(0xFFFFFFFFu, v[0], 1);
+}
+
+// Moments of an arbitrary state (Eqs. densita..sforzi), one CTA per cell, all
+// sums in FP64.  mu (nullable): the pending corrections of a state stored as
+// h_c (8 floats per cell), applied in FP32 as a state copy applies them.
+//
+// Bound by the FP64 pipe (about two operations per cycle and SM): the sums
+// over v_x are taken first at fixed (v_y, v_z), so a node costs a conversion
+// and three multiply-adds, against about 25 operations when every node was
+// multiplied into all ten sums.  Sixteen cavities of 32^2..128^2 cells and
+// 16^3..24^3 nodes: 29.0 ms before (ncu, all sixteen); the pass of six batch steps
+// that reads every state and its moments went from 62.4 to 39.8 ms with this
+// and the one-pass state copy.
+constexpr int kMomThreads = 256;
+template <typename R>
+__global__ void __launch_bounds__(kMomThreads) k_moments(Geo g, const R *__restrict__ h, double *__restrict__ mom,
+                                                         const float *__restrict__ mu = nullptr)
+{
+    constexpr int W = kMomThreads / 32, U = 8;
+    __shared__ double sA[kMaxN], sAv[kMaxN], sAv2[kMaxN], sv[kMaxN];
+    __shared__ float svf[kMaxN];
+    __shared__ double part[W][16];
+    const int N = g.nv, N2 = N * N, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int i = t; i < N; i += kMomThreads) {
+        const double v = g.axv[i], A = g.axA[i];
+        sA[i] = A;
+        sAv[i] = A * v;
+        sAv2[i] = A * v * v;
+        sv[i] = v;
+        svf[i] = (float)v;
+    }
+    const float epsf = g.epsf;
+    for (int c = blockIdx.x; c < g.nr; c += gridDim.x) {
+        float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        if (mu)
+            for (int k = 0; k < 5; ++k) m[k] = mu[(int64_t)c * 8 + k];
+        __syncthreads();
+        double mo[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) mo[k] = 0.0;
+        const R *src = h + (int64_t)c * g.nvt;
+        for (int p = t; p < N2; p += kMomThreads) {
+            const int jy = p / N, jz = p - jy * N;
+            const float vyf = svf[jy], vzf = svf[jz];
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+            for (int j0 = 0; j0 < N; j0 += U) {
+                R x[U];
+#pragma unroll
+                for (int k = 0; k < U; ++k) x[k] = j0 + k < N ? src[(int64_t)(j0 + k) * N2 + p] : R(0);
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const int jx = j0 + k;
+                    if (jx >= N) break;
+                    if constexpr (sizeof(R) == 4) {
+                        if (mu) x[k] = state_corr(x[k], state_kappa(m, svf[jx], vyf, vzf), epsf);
+                    }
+                    const double n = (double)x[k];
+                    s0 += sA[jx] * n;
+                    s1 += sAv[jx] * n;
+                    s2 += sAv2[jx] * n;
+                }
+            }
+            const double vy = sv[jy], vz = sv[jz], Ayz = sA[jy] * sA[jz];
+            const double n0 = Ayz * s0, n1 = Ayz * s1, ny = vy * n0, nz = vz * n0;
+            mo[0] += n0;
+            mo[1] += n1;
+            mo[2] += ny;
+            mo[3] += nz;
+            mo[4] += Ayz * s2;
+            mo[5] += vy * ny;
+            mo[6] += vz * nz;
+            mo[7] += vy * n1;
+            mo[8] += vz * n1;
+            mo[9] += vy * nz;
+        }
+        const double r = warp_reduce_scatter16(mo);
+        if (!(lane & 1)) part[warp][lane >> 1] = r;
+        __syncthreads();
+        if (t < 16) {
+            double s = 0.0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) s += part[w][t];
+            part[0][t] = s;
+        }
+        __syncwarp();
+        if (t == 0) {
+            const double *q = part[0], e = g.eps;
+            double rho = q[0], n = 1.0 + e * rho;
+            double u[3] = {q[1] / n, q[2] / n, q[3] / n};
             double *o = mom + (int64_t)c * 11;
             o[0] = rho;
             o[1] = u[0];
             o[2] = u[1];
             o[3] = u[2];
-            o[4] = ((2.0 / 3.0) * (m[4] + m[5] + m[6]) - rho) / n -
+            o[4] = ((2.0 / 3.0) * (q[4] + q[5] + q[6]) - rho) / n -
                    (2.0 * e / 3.0) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
             const int pa[6] = {0, 1, 2, 0, 0, 1}, pb[6] = {0, 1, 2, 1, 2, 2};
-            const double m2[6] = {m[4], m[5], m[6], m[7], m[8], m[9]};
-            for (int k = 0; k < 6; ++k) o[5 + k] = 2.0 * m2[k] - 2.0 * e * n * u[pa[k]] * u[pb[k]];
+            for (int k = 0; k < 6; ++k) o[5 + k] = 2.0 * q[4 + k] - 2.0 * e * n * u[pa[k]] * u[pb[k]];
         }
-        __syncthreads();
     }
 }
 

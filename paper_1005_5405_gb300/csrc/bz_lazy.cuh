@@ -551,12 +551,6 @@ static __global__ void k_lz_fb_plan(int nt, int N, const int *__restrict__ meta,
     if (l < nt) lz_fb_plan_one(l, N, idx, pa, pidx16, pa16, count);
 }
 
-// The correction of a stored node value: h = h_c + (1 + eps h_c) kappa.
-__device__ __forceinline__ float lz_corr(float hc, float kappa, float eps)
-{
-    return fmaf(eps * hc, kappa, hc + kappa);
-}
-
 // h <- h_c + (1 + eps h_c)(mu_c . psi_j) for every node (in place allowed:
 // hout may be hin, so neither is restrict-qualified); mu_zero (nullable) is
 // then cleared, and mu_used (nullable; may be mu) gets each cell's
@@ -583,13 +577,11 @@ static __global__ void k_lz_materialize(Geo g, const int *__restrict__ skip_unle
         for (int o = threadIdx.x; o < (int)plane; o += blockDim.x) {
             const int jx = o / Q, q = o % Q, jy = q / nq, jz = 4 * (q % nq);
             const float vx = sv[jx], vy = sv[jy];
-            const float base = smu[0] + smu[1] * vx + smu[2] * vy + smu[4] * (vx * vx + vy * vy);
             float4 h = src[o];
             float *hp = &h.x;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const float vz = sv[jz + i];
-                hp[i] = lz_corr(hp[i], base + smu[3] * vz + smu[4] * vz * vz, eps);
+                hp[i] = state_corr(hp[i], state_kappa(smu, vx, vy, sv[jz + i]), eps);
             }
             dst[o] = h;
         }
