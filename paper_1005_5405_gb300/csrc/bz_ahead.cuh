@@ -26,7 +26,7 @@ struct AheadPlans {
     int *wpre;                      // K x nvt/32
     int *meta;                      // K x kLzMetaSize
     int *count, *cursor, *rowend;   // K x nvt
-    int *dest0;                     // K x kLzRoleT
+    int *dest0;                     // K x kLzCollT
     uint2 *rec;                     // K x recn term records
     int64_t recn;
     unsigned long long *cnt;        // K x 2: samples with a node outside the box, near a face
@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(1024) k_ahead_lscan(AheadPlans A, int64_t step
 {
     const int s = ahead_slot(A, step0, blockIdx.x);
     const int64_t v = (int64_t)s * A.nvt;
-    lz_lscan_block(kLzRoleT, A.osh, A.count + v, A.cursor + v, A.rowend + v, A.meta + s * kLzMetaSize,
-                   A.rec + s * A.recn, A.dest0 + s * kLzRoleT);
+    lz_lscan_block(kLzCollT, A.osh, A.count + v, A.cursor + v, A.rowend + v, A.meta + s * kLzMetaSize,
+                   A.rec + s * A.recn, A.dest0 + s * kLzCollT);
 }
 
 __global__ void k_ahead_lfill(AheadPlans A, int64_t step0)
@@ -101,8 +101,8 @@ __global__ void k_ahead_lfill(AheadPlans A, int64_t step0)
     if (l >= A.nt) return;
     const int s = ahead_slot(A, step0, blockIdx.y);
     const int64_t t = (int64_t)s * A.nt, v = (int64_t)s * A.nvt;
-    lz_lfill_one(l, kLzRoleT, A.osh, A.qc + t, A.pa + t, A.cursor + v, A.rowend + v,
-                 A.meta + s * kLzMetaSize, A.rec + s * A.recn, A.dest0 + s * kLzRoleT);
+    lz_lfill_one(l, kLzCollT, A.osh, A.qc + t, A.pa + t, A.cursor + v, A.rowend + v,
+                 A.meta + s * kLzMetaSize, A.rec + s * A.recn, A.dest0 + s * kLzCollT);
 }
 
 // The plan of step `step` into the arrays the step reads, and its counters
@@ -130,10 +130,10 @@ __device__ __forceinline__ void ahead_take(const AheadPlans &A, int64_t step, in
         wpre[i] = A.wpre[w0 + i];
     }
     for (int64_t i = i0; i < M; i += stride) act[i] = A.act[v0 + i];
-    const int64_t nrec = min((int64_t)C * kLzRoleT, A.recn);
+    const int64_t nrec = min((int64_t)C * kLzCollT, A.recn);
     const uint2 *sr = A.rec + s * A.recn;
     for (int64_t i = i0; i < nrec; i += stride) rec[i] = sr[i];
-    for (int64_t i = i0; i < kLzRoleT; i += stride) dest0[i] = A.dest0[(int64_t)s * kLzRoleT + i];
+    for (int64_t i = i0; i < kLzCollT; i += stride) dest0[i] = A.dest0[(int64_t)s * kLzCollT + i];
     if (i0 < kLzMetaSize) meta[i0] = sm[i0];
     if (i0 == 0 && stats) {
         stats[1] += A.cnt[2 * s];

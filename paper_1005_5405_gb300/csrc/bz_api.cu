@@ -137,7 +137,7 @@ struct bz_handle {
     int *lz_dest0 = nullptr;
     uint32_t *lz_mask = nullptr;
     uint2 *lz_rec = nullptr;
-    int lz_mcap = 0, lz_G = 0, lz_T = 0, lz_grid = 0, lz_mprobe = 0;
+    int lz_mcap = 0, lz_G = 0, lz_T = 0, lz_grid = 0, lz_mprobe = 0, lz_stages = 0;
     int lz_cmax = 0, lz_order_tpb = 0;     // bank-aware ordering of the term runs (1: on)
     bool lz_tma = false;                   // streaming sources by bulk copies (G = 4 only)
     // Plans built ahead (bz_ahead.cuh): K slots, covering steps [ahead_lo, ahead_hi).
@@ -423,48 +423,49 @@ double lz_monomial(int k, double x, double y, double z)
 // the kernel that reads it at run time); stretched grids (per-cell Courant
 // factors) have their own instances, specialised for 20 nodes per axis (the
 // paper's stretched cavities) and run-time lengths otherwise.
-int lz_nv_key(const bz_handle *H) { return H->stretched ? (H->g.nv == 20 ? -20 : -1) : (H->g.nv == 32 || H->g.nv == 20 ? H->g.nv : 0); }
+int lz_nv_key(const bz_handle *H) { return H->stretched ? (H->g.nv == 20 ? -20 : -1) : H->g.nv; }
 
-template <int G, int NV, bool SX, bool TMA = false>
-bz_status setup_lz_one(bz_handle *H, size_t smem, int *occ)
+// Calls f with the k_lz instance of a handle: G cells per group, the axis
+// length as a constant where it has an instance, stretched cells, the
+// streaming threads, the bulk-copy ring.
+template <int G, int ST, typename F>
+auto with_lz_kernel(const bz_handle *H, F f)
 {
-    BZ_CUDA(bz_allow_max_smem(bzk::k_lz<G, NV, SX, TMA>, H->smem_optin));
-    BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, bzk::k_lz<G, NV, SX, TMA>, H->lz_T, smem));
-    return BZ_OK;
-}
-
-template <int G>
-bz_status setup_lz_kernel(bz_handle *H, size_t smem, int *occ)
-{
-    if (G == 4 && H->lz_tma && lz_nv_key(H) >= 0)
-        return lz_nv_key(H) == 32 ? setup_lz_one<4, 32, false, true>(H, smem, occ)
-                                  : setup_lz_one<4, 0, false, true>(H, smem, occ);
-    switch (lz_nv_key(H)) {
-    case 32: return setup_lz_one<G, 32, false>(H, smem, occ);
-    case 20: return setup_lz_one<G, 20, false>(H, smem, occ);
-    case -1: return setup_lz_one<G, 0, true>(H, smem, occ);
-    case -20: return setup_lz_one<G, 20, true>(H, smem, occ);
-    default: return setup_lz_one<G, 0, false>(H, smem, occ);
+    if constexpr (G == 4 && ST == 256) {
+        if (H->lz_tma && lz_nv_key(H) >= 0)
+            return lz_nv_key(H) == 32 ? f(bzk::k_lz<4, 32, false, 256, true>) : f(bzk::k_lz<4, 0, false, 256, true>);
     }
+    if constexpr (G == 4 && ST == 512) {
+        if (lz_nv_key(H) == 24) return f(bzk::k_lz<4, 24, false, 512>);
+    } else if constexpr (G == 4) {
+        switch (lz_nv_key(H)) {
+        case 32: return f(bzk::k_lz<4, 32, false, ST>);
+        case 28: return f(bzk::k_lz<4, 28, false, ST>);
+        case 20: return f(bzk::k_lz<4, 20, false, ST>);
+        case 16: return f(bzk::k_lz<4, 16, false, ST>);
+        case -20: return f(bzk::k_lz<4, 20, true, ST>);
+        }
+    }
+    return H->stretched ? f(bzk::k_lz<G, 0, true, ST>) : f(bzk::k_lz<G, 0, false, ST>);
 }
 
-template <int G>
+bz_status setup_lz_kernel(bz_handle *H, int G, int ST, size_t smem, int *occ)
+{
+    auto set = [&](auto *k) -> bz_status {
+        BZ_CUDA(bz_allow_max_smem(k, H->smem_optin));
+        BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, bzk::lz_threads(ST), smem));
+        return BZ_OK;
+    };
+    if (ST == 512) return with_lz_kernel<4, 512>(H, set);
+    return G == 4 ? with_lz_kernel<4, 256>(H, set) : with_lz_kernel<2, 256>(H, set);
+}
+
 void launch_lz_kernel(bz_handle *H, const bzk::LzArgs &a, cudaStream_t s)
 {
-    if (G == 4 && H->lz_tma && lz_nv_key(H) >= 0) {
-        if (lz_nv_key(H) == 32)
-            bzk::k_lz<4, 32, false, true><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a);
-        else
-            bzk::k_lz<4, 0, false, true><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a);
-        return;
-    }
-    switch (lz_nv_key(H)) {
-    case 32: bzk::k_lz<G, 32, false><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); break;
-    case 20: bzk::k_lz<G, 20, false><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); break;
-    case -1: bzk::k_lz<G, 0, true><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); break;
-    case -20: bzk::k_lz<G, 20, true><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); break;
-    default: bzk::k_lz<G, 0, false><<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); break;
-    }
+    auto go = [&](auto *k) { k<<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); };
+    if (H->lz_T == bzk::lz_threads(512)) with_lz_kernel<4, 512>(H, go);
+    else if (H->lz_G == 4) with_lz_kernel<4, 256>(H, go);
+    else with_lz_kernel<2, 256>(H, go);
 }
 
 // Decide whether the active-node path applies (FP32 fast path, at most 32
@@ -481,8 +482,7 @@ bz_status configure_lazy(bz_handle *H)
     if (force && (strcmp(force, "generic") == 0 || strcmp(force, "cell4") == 0)) return BZ_OK;
     if (!H->fast || g.nv > bzk::kLzMaxN || g.nv % 4 != 0 || g.nvt % 32 != 0) return BZ_OK;
     const int N = g.nv, nvt = g.nvt, nt = g.nt;
-    const int P4 = bzk::lz_planes4(N);
-    if (P4 == 0) return BZ_OK;
+    if (bzk::lz_planes4(N, 256) == 0) return BZ_OK;
     const size_t mub = sizeof(float) * 8 * (size_t)g.nr;
     BZ_TRY(dalloc(&H->mu[0], mub));
     BZ_TRY(dalloc(&H->mu[1], mub));
@@ -528,33 +528,40 @@ bz_status configure_lazy(bz_handle *H)
     if (const char *mc = getenv("BZ_LAZY_MCAP")) mcap = std::max(1, std::min(nvt, atoi(mc)));
     if (const char *tm = getenv("BZ_LAZY_TMA")) H->lz_tma = atoi(tm) != 0;
 
-    // One CTA of two 256-thread roles per SM; the largest group of cells
-    // whose shared memory fits.
-    H->lz_T = bzk::kLzThreads;
+    // One CTA per SM: the largest group of cells whose shared memory fits,
+    // and 512 streaming threads where they pay (bz_lazy.cuh).
     bool ok = false;
     const char *force_g = getenv("BZ_LAZY_G");
-    for (int G : {4, 2}) {
-        if (force_g && atoi(force_g) != G) continue;
-        // Term records address a compact array with 16-bit byte offsets.
-        if ((size_t)mcap * 4 * G > 65535) continue;
-        const size_t smem = bzk::lz_offsets(nvt, mcap, G).end;
-        if (smem > (size_t)H->smem_optin) continue;
-        int occ = 0;
-        if (G == 4) BZ_TRY(setup_lz_kernel<4>(H, smem, &occ));
-        else BZ_TRY(setup_lz_kernel<2>(H, smem, &occ));
-        if (occ < 1) continue;
-        H->lz_G = G;
-        H->lz_smem = smem;
-        H->lz_grid = std::min((g.nr + G - 1) / G, H->nsm);
-        if (const char *c = getenv("BZ_LAZY_CTAS")) H->lz_grid = std::max(1, std::min(H->lz_grid, atoi(c)));
-        ok = true;
-        break;
+    const char *force_st = getenv("BZ_LAZY_ST");
+    for (const int ST : {512, 256}) {
+        for (const int G : {4, 2}) {
+            if (ok || (force_g && atoi(force_g) != G) || (force_st && atoi(force_st) != ST)) continue;
+            if (ST == 512 && (G != 4 || (!force_st && bzk::lz_stream_threads(N) != 512) || H->lz_tma)) continue;
+            // Term records address a compact array with 16-bit byte offsets.
+            if ((size_t)mcap * 4 * G > 65535) continue;
+            // As many streaming stages as fit (the copies in flight per SM).
+            const int S = bzk::lz_planes4(N, ST) * (N * N / 4);
+            int stages = bzk::kLzMaxStages;
+            while (stages >= 3 && bzk::lz_offsets(nvt, mcap, G, stages, S).end > (size_t)H->smem_optin) --stages;
+            if (stages < 3) continue;
+            const size_t smem = bzk::lz_offsets(nvt, mcap, G, stages, S).end;
+            int occ = 0;
+            BZ_TRY(setup_lz_kernel(H, G, ST, smem, &occ));
+            if (occ < 1) continue;
+            H->lz_G = G;
+            H->lz_T = bzk::lz_threads(ST);
+            H->lz_smem = smem;
+            H->lz_stages = stages;
+            H->lz_grid = std::min((g.nr + G - 1) / G, H->nsm);
+            if (const char *c = getenv("BZ_LAZY_CTAS")) H->lz_grid = std::max(1, std::min(H->lz_grid, atoi(c)));
+            ok = true;
+        }
     }
     if (!ok) return BZ_OK;
     H->lz_mcap = mcap;
     // Bank-aware ordering of the term runs: one warp per phase group of
     // runs, with their records staged in shared memory.
-    H->lz_cmax = ((4 * nt + bzk::kLzRoleT - 1) / bzk::kLzRoleT + 7) / 8 * 8;
+    H->lz_cmax = ((4 * nt + bzk::kLzCollT - 1) / bzk::kLzCollT + 7) / 8 * 8;
     {
         const int nb = H->lz_G == 4 ? 8 : 16;
         H->lz_chunk = std::min(H->lz_cmax, 64);
@@ -582,8 +589,8 @@ bz_status configure_lazy(bz_handle *H)
     BZ_TRY(dalloc(&H->lz_count, sizeof(int) * (size_t)nvt));
     BZ_TRY(dalloc(&H->lz_cursor, sizeof(int) * (size_t)nvt));
     BZ_TRY(dalloc(&H->lz_rowend, sizeof(int) * (size_t)nvt));
-    BZ_TRY(dalloc(&H->lz_dest0, sizeof(int) * (size_t)bzk::kLzRoleT));
-    BZ_TRY(dalloc(&H->lz_rec, sizeof(uint2) * ((size_t)4 * nt + (size_t)8 * bzk::kLzRoleT)));
+    BZ_TRY(dalloc(&H->lz_dest0, sizeof(int) * (size_t)bzk::kLzCollT));
+    BZ_TRY(dalloc(&H->lz_rec, sizeof(uint2) * ((size_t)4 * nt + (size_t)8 * bzk::kLzCollT)));
     BZ_CUDA(cudaMemset(H->lz_count, 0, sizeof(int) * (size_t)nvt));
     // Plans of K steps built ahead at a time (BZ_LAZY_AHEAD=K sets the
     // count, 0 builds each step's plan in the step), their term order over
@@ -602,7 +609,7 @@ bz_status configure_lazy(bz_handle *H)
         H->ahead_K = 32;
         if (H->lz_order_tpb > 0) {
             const int nch = (H->lz_cmax + H->ahead_chunk - 1) / H->ahead_chunk;
-            const int64_t per = (int64_t)(bzk::kLzRoleT / nb) * nch;       // CTAs per plan
+            const int64_t per = (int64_t)(bzk::kLzCollT / nb) * nch;       // CTAs per plan
             int occ = 0;
             const size_t osm = bzk::lz_order_smem(H->ahead_chunk, nb);
             BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -623,7 +630,7 @@ bz_status configure_lazy(bz_handle *H)
         A.nvt = nvt;
         A.mcap = mcap;
         A.osh = H->lz_G == 4 ? 4 : 3;
-        A.recn = (int64_t)4 * nt + (int64_t)8 * bzk::kLzRoleT;
+        A.recn = (int64_t)4 * nt + (int64_t)8 * bzk::kLzCollT;
         const size_t k = (size_t)K;
         BZ_TRY(dalloc(&A.idx, sizeof(int4) * k * nt));
         BZ_TRY(dalloc(&A.pa, sizeof(bzk::PlanA<float, int>) * k * nt));
@@ -637,7 +644,7 @@ bz_status configure_lazy(bz_handle *H)
         BZ_TRY(dalloc(&A.count, sizeof(int) * k * nvt));
         BZ_TRY(dalloc(&A.cursor, sizeof(int) * k * nvt));
         BZ_TRY(dalloc(&A.rowend, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.dest0, sizeof(int) * k * bzk::kLzRoleT));
+        BZ_TRY(dalloc(&A.dest0, sizeof(int) * k * bzk::kLzCollT));
         BZ_TRY(dalloc(&A.rec, sizeof(uint2) * k * (size_t)A.recn));
         BZ_TRY(dalloc(&A.cnt, sizeof(unsigned long long) * 2 * k));
         BZ_CUDA(cudaMemset(A.flag, 0, sizeof(int) * k * nvt));
@@ -706,11 +713,11 @@ bz_status ensure_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt)
     if (H->lz_order_tpb > 0) {
         const int ch = H->ahead_chunk, nch = (H->lz_cmax + ch - 1) / ch, z0 = (int)(n % K);
         if (H->lz_G == 4)
-            bzk::k_lz_order<8><<<dim3(bzk::kLzRoleT / 8, nch, K), 32, bzk::lz_order_smem(ch, 8), s>>>(
-                bzk::kLzRoleT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
+            bzk::k_lz_order<8><<<dim3(bzk::kLzCollT / 8, nch, K), 32, bzk::lz_order_smem(ch, 8), s>>>(
+                bzk::kLzCollT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
         else
-            bzk::k_lz_order<16><<<dim3(bzk::kLzRoleT / 16, nch, K), 32, bzk::lz_order_smem(ch, 16), s>>>(
-                bzk::kLzRoleT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
+            bzk::k_lz_order<16><<<dim3(bzk::kLzCollT / 16, nch, K), 32, bzk::lz_order_smem(ch, 16), s>>>(
+                bzk::kLzCollT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
         BZ_LAUNCHED(H);
     }
     H->ahead_lo = n;
@@ -752,11 +759,11 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
         BZ_LAUNCHED(H);
         bzk::k_lz_remap<<<pg, pb, 0, sp>>>(g.nt, H->lz_idx, H->lz_cidx, H->lz_qc, H->lz_count);
         BZ_LAUNCHED(H);
-        bzk::k_lz_lscan<<<1, 1024, 0, sp>>>(bzk::kLzRoleT, H->lz_G == 4 ? 4 : 3, H->lz_count,
+        bzk::k_lz_lscan<<<1, 1024, 0, sp>>>(bzk::kLzCollT, H->lz_G == 4 ? 4 : 3, H->lz_count,
                                            H->lz_cursor, H->lz_rowend,
                                            H->lz_meta, H->lz_rec, H->lz_dest0);
         BZ_LAUNCHED(H);
-        bzk::k_lz_lfill<<<pg, pb, 0, sp>>>(g.nt, bzk::kLzRoleT, H->lz_G == 4 ? 4 : 3, H->lz_qc, H->lz_pa,
+        bzk::k_lz_lfill<<<pg, pb, 0, sp>>>(g.nt, bzk::kLzCollT, H->lz_G == 4 ? 4 : 3, H->lz_qc, H->lz_pa,
                                           H->lz_cursor, H->lz_rowend, H->lz_meta, H->lz_rec,
                                           H->lz_dest0);
         BZ_LAUNCHED(H);
@@ -766,11 +773,11 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
             BZ_CUDA(cudaEventRecord(H->lz_mid, sp));
             const int nch = (H->lz_cmax + H->lz_chunk - 1) / H->lz_chunk;
             if (H->lz_G == 4)
-                bzk::k_lz_order<8><<<dim3(bzk::kLzRoleT / 8, nch), 32, bzk::lz_order_smem(H->lz_chunk, 8), sp>>>(
-                    bzk::kLzRoleT, H->lz_cmax, H->lz_chunk, H->lz_meta, H->lz_rec);
+                bzk::k_lz_order<8><<<dim3(bzk::kLzCollT / 8, nch), 32, bzk::lz_order_smem(H->lz_chunk, 8), sp>>>(
+                    bzk::kLzCollT, H->lz_cmax, H->lz_chunk, H->lz_meta, H->lz_rec);
             else
-                bzk::k_lz_order<16><<<dim3(bzk::kLzRoleT / 16, nch), 32, bzk::lz_order_smem(H->lz_chunk, 16), sp>>>(
-                    bzk::kLzRoleT, H->lz_cmax, H->lz_chunk, H->lz_meta, H->lz_rec);
+                bzk::k_lz_order<16><<<dim3(bzk::kLzCollT / 16, nch), 32, bzk::lz_order_smem(H->lz_chunk, 16), sp>>>(
+                    bzk::kLzCollT, H->lz_cmax, H->lz_chunk, H->lz_meta, H->lz_rec);
             BZ_LAUNCHED(H);
         }
     }
@@ -799,6 +806,7 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
         a.wpre = H->lz_wpre;
         a.act = H->lz_act;
         a.mcap = H->lz_mcap;
+        a.stages = H->lz_stages;
         for (int k = 0; k < bzk::kLzX; ++k) a.e0[k] = H->lz_e0[k];
         a.clk = H->prof_clk;
         a.stats = H->stats;
@@ -810,12 +818,11 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
         // bounded waits; the step's result is then invalid).
         if (const char *tt = getenv("BZ_LAZY_TMA_TIMEOUT_TEST")) a.tx_excess = atoi(tt) != 0 ? 16 : 0;
         a.nostream = nostream ? 1 : 0;
-        // Below 32^3 velocities the streaming of a group takes longer than
-        // its collision terms: the collision warps start the increment sums.
-        a.early_tail = g.nv < 32 ? 1 : 0;
+        // The streaming of a group takes longer than its collision terms: the
+        // collision warps start the increment sums.
+        a.early_tail = 1;
         if (const char *et = getenv("BZ_LAZY_EARLY_TAIL")) a.early_tail = atoi(et) != 0 ? 1 : 0;
-        if (H->lz_G == 4) launch_lz_kernel<4>(H, a, s);
-        else launch_lz_kernel<2>(H, a, s);
+        launch_lz_kernel(H, a, s);
         BZ_LAUNCHED(H);
     }
     {
@@ -1839,7 +1846,7 @@ struct bz_batch {
     int *d_next = nullptr;                  // one claim counter per velocity grid
     int nseg = 0;
     size_t lz_smem = 0;
-    struct LzClass { int nv, seg0, nseg; size_t smem; };
+    struct LzClass { int nv, ST, seg0, nseg; size_t smem; };
     std::vector<LzClass> lz_classes;        // the segments of each velocity grid
     cudaStream_t lz_side = nullptr;         // the sample plans run here, beside the walls
     cudaEvent_t lz_fork = nullptr, lz_join = nullptr;
@@ -1982,6 +1989,14 @@ bz_status batch_correct_in_place(bz_batch *B, int i, cudaStream_t s)
     BZ_CUDA(cudaGetLastError());
     BZ_CUDA(cudaMemsetAsync(h->mu[b], 0, sizeof(float) * 8 * (size_t)h->g.nr, s));
     return BZ_OK;
+}
+
+// Calls f with the batch kernel instance of a velocity-grid class.
+template <typename F>
+auto with_kbl_lz(int nv, int ST, F f)
+{
+    if (ST == 512) return nv == 24 ? f(bzk::kbl_lz<24, 512>) : f(bzk::kbl_lz<0, 512>);
+    return nv == 20 ? f(bzk::kbl_lz<20, 256>) : nv == 16 ? f(bzk::kbl_lz<16, 256>) : f(bzk::kbl_lz<0, 256>);
 }
 
 // One fan-out step: fork to the branches, each instance's active-node step
@@ -2127,12 +2142,9 @@ bz_status lz_batch_launch(bz_batch *B, cudaStream_t s, bool advance)
         int *nx = B->d_next + k;
         const cudaStream_t sk = k == 0 ? s : B->lz_cls_s[k - 1];
         if (k > 0) BZ_CUDA(cudaStreamWaitEvent(sk, B->lz_go, 0));
-        switch (c.nv) {
-        case 24: bzk::kbl_lz<24><<<B->nsm, bzk::kLzThreads, c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx); break;
-        case 20: bzk::kbl_lz<20><<<B->nsm, bzk::kLzThreads, c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx); break;
-        case 16: bzk::kbl_lz<16><<<B->nsm, bzk::kLzThreads, c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx); break;
-        default: bzk::kbl_lz<0><<<B->nsm, bzk::kLzThreads, c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx); break;
-        }
+        with_kbl_lz(c.nv, c.ST, [&](auto *kern) {
+            kern<<<B->nsm, bzk::lz_threads(c.ST), c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx);
+        });
         if (k > 0) BZ_CUDA(cudaEventRecord(B->lz_cls_done[k - 1], sk));
     }
     for (size_t k = 1; k < nc; ++k) BZ_CUDA(cudaStreamWaitEvent(s, B->lz_cls_done[k - 1], 0));
@@ -2204,42 +2216,49 @@ bz_status lz_batch_prepare(bz_batch *B)
             a.wpre = h->lz_wpre;
             a.act = h->lz_act;
             a.mcap = h->lz_mcap;
+            a.stages = h->lz_stages;
             for (int k = 0; k < bzk::kLzX; ++k) a.e0[k] = h->lz_e0[k];
             a.stats = h->stats;
-            a.early_tail = h->g.nv < 32 ? 1 : 0;
+            a.early_tail = 1;
         }
-        smem = std::max(smem, (size_t)bzk::lz_offsets(h->g.nvt, h->lz_mcap, 4).end);
+        smem = std::max(smem, (size_t)h->lz_smem);
         order[i] = i;
     }
     // Segments of about 32 groups: R strided lanes r, r + R, ... of each
     // instance's groups, the instances with the largest velocity grids (the
     // costliest groups) first.
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-        return B->inst[x]->g.nv > B->inst[y]->g.nv;
+        return B->inst[x]->g.nv != B->inst[y]->g.nv ? B->inst[x]->g.nv > B->inst[y]->g.nv
+                                                    : B->inst[x]->lz_T > B->inst[y]->lz_T;
     });
     std::vector<int4> segs;
     B->lz_classes.clear();
     for (int i : order) {
         const int nv = B->inst[i]->g.nv;
         const int key = nv == 24 || nv == 20 || nv == 16 ? nv : 0;
-        if (B->lz_classes.empty() || B->lz_classes.back().nv != key)
-            B->lz_classes.push_back({key, (int)segs.size(), 0, 0});
+        const int ST = B->inst[i]->lz_T - bzk::kLzCollT;
+        if (B->lz_classes.empty() || B->lz_classes.back().nv != key || B->lz_classes.back().ST != ST)
+            B->lz_classes.push_back({key, ST, (int)segs.size(), 0, 0});
         auto &c = B->lz_classes.back();
-        c.smem = std::max(c.smem, (size_t)bzk::lz_offsets(B->inst[i]->g.nvt, B->inst[i]->lz_mcap, 4).end);
+        c.smem = std::max(c.smem, (size_t)B->inst[i]->lz_smem);
         const int ng = (B->inst[i]->g.nr + 3) / 4, R = std::max(1, (ng + 31) / 32);
         for (int r = 0; r < R && r < ng; ++r) segs.push_back(make_int4(i, r, (ng - 1 - r) / R + 1, R));
         c.nseg = (int)segs.size() - c.seg0;
     }
     bz_handle *h0 = B->inst[0];
-    BZ_CUDA(bz_allow_max_smem(bzk::kbl_lz<24>, h0->smem_optin));
-    BZ_CUDA(bz_allow_max_smem(bzk::kbl_lz<20>, h0->smem_optin));
-    BZ_CUDA(bz_allow_max_smem(bzk::kbl_lz<16>, h0->smem_optin));
-    BZ_CUDA(bz_allow_max_smem(bzk::kbl_lz<0>, h0->smem_optin));
+    for (const auto &c : B->lz_classes) {
+        int occ = 0;
+        BZ_TRY(with_kbl_lz(c.nv, c.ST, [&](auto *kern) -> bz_status {
+            BZ_CUDA(bz_allow_max_smem(kern, h0->smem_optin));
+            BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, bzk::lz_threads(c.ST), c.smem));
+            return BZ_OK;
+        }));
+        if (occ < 1) return BZ_OK;
+    }
     BZ_CUDA(bz_allow_max_smem(bzk::kbl_fb_cell4, h0->smem_optin));
-    int occ = 0, occ4 = 0;
-    BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bzk::kbl_lz<0>, bzk::kLzThreads, smem));
+    int occ4 = 0;
     BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ4, bzk::kbl_fb_cell4, 512, B->smem));
-    if (occ < 1 || occ4 < 1) return BZ_OK;
+    if (occ4 < 1) return BZ_OK;
     BZ_TRY(dalloc(&B->d_lzinst, sizeof(bzk::LzInst) * n));
     BZ_TRY(dalloc(&B->d_segs, sizeof(int4) * segs.size()));
     BZ_TRY(dalloc(&B->d_next, sizeof(int) * B->lz_classes.size()));

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(1024) kbl_lscan(const LzInst *__restrict__ ins
 {
     const LzInst &b = inst[blockIdx.x];
     const LzArgs &a = b.a[0];
-    lz_lscan_block(kLzRoleT, 4, b.count, b.cursor, b.rowend, const_cast<int *>(a.meta),
+    lz_lscan_block(kLzCollT, 4, b.count, b.cursor, b.rowend, const_cast<int *>(a.meta),
                    const_cast<uint2 *>(a.rec), const_cast<int *>(a.dest0));
 }
 
@@ -284,7 +284,7 @@ __global__ void kbl_lfill(const LzInst *__restrict__ inst, const int *__restrict
     const int i = inst_of(samp_pre, n, k);
     const LzInst &b = inst[i];
     const LzArgs &a = b.a[0];
-    lz_lfill_one(k - samp_pre[i], kLzRoleT, 4, b.qc, b.pa, b.cursor, b.rowend, a.meta,
+    lz_lfill_one(k - samp_pre[i], kLzCollT, 4, b.qc, b.pa, b.cursor, b.rowend, a.meta,
                  const_cast<uint2 *>(a.rec), const_cast<int *>(a.dest0));
 }
 
@@ -295,8 +295,8 @@ __global__ void kbl_lfill(const LzInst *__restrict__ inst, const int *__restrict
 // (neighbouring cells are streamed together and their slabs shared in L2).
 // Groups of four cells; one launch per velocity grid (NV: its axis length as
 // a compile-time constant, 0 read at run time), sized for that grid.
-template <int NV>
-__global__ void __launch_bounds__(kLzThreads, 1) kbl_lz(const LzInst *__restrict__ inst,
+template <int NV, int ST>
+__global__ void __launch_bounds__(lz_threads(ST), 1) kbl_lz(const LzInst *__restrict__ inst,
                                                        const int4 *__restrict__ segs, int nseg,
                                                        int *__restrict__ next)
 {
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) kbl_lz(const LzInst *__restrict
             s_a = b.a[*b.step & 1];
         }
         __syncthreads();
-        lz_run<4, NV, false>(s_g, s_a, smem_raw, q.y, q.w, q.z);
+        lz_run<4, NV, false, ST>(s_g, s_a, smem_raw, q.y, q.w, q.z);
     }
 }
 

@@ -44,12 +44,22 @@ namespace bzk {
 
 constexpr int kLzMono = 26;        // monomial sums per cell
 constexpr int kLzX = 30;           // with v^2, v_x v^2, v_y v^2, v_z v^2
-constexpr int kLzRoleT = 256;      // threads of each role: streaming, collision
-constexpr int kLzThreads = 2 * kLzRoleT;
-constexpr int kLzRoleWarps = kLzRoleT / 32;
+// Threads of the collision role, and of the streaming role (ST, a template
+// argument of the kernel).  256 streaming threads leave 128 registers a
+// thread; with 512 (80 registers) a stage covers up to twice the jx-planes or
+// more, so that the streaming of a cell takes fewer stages, but each stage of
+// the ring is larger.  512 pay only where they keep a larger share of the
+// threads busy: at 24 nodes per axis a stage has 432 quads (3 planes) against
+// 144 (1 plane of 256 threads).  k_lz with 256 / 512 streaming threads: 128^2 x
+// 24^3 989 / 821 us; 128^2 x 20^3 580 / 598, 128^2 x 16^3 407 / 480, 96^2 x 28^3 757 /
+// 780, 128^2 x 12^3 284 / 346 us.
+constexpr int kLzCollT = 256;
+constexpr int kLzMaxStreamT = 512;
+__host__ __device__ constexpr int lz_threads(int ST) { return ST + kLzCollT; }
+constexpr int kLzDParts = 8;       // slots of the increment sums per cell
 constexpr int kLzMaxG = 4;         // cells per CTA group
-constexpr int kLzMaxN = 32;        // velocity nodes per axis (N^2 / 4 <= kLzRoleT)
-constexpr int kLzStages = 5;       // streaming stages staged per thread
+constexpr int kLzMaxN = 32;        // velocity nodes per axis (N^2 / 4 <= 256)
+constexpr int kLzMaxStages = 5;    // streaming stages staged per thread (at least 2)
 constexpr unsigned long long kLzWaitNs = 1000000000ull;   // an mbarrier wait gives up after 1 s
 
 // meta layout: [0] M, [1] overflow (M > mcap), [2] E (terms of the step),
@@ -57,15 +67,23 @@ constexpr unsigned long long kLzWaitNs = 1000000000ull;   // an mbarrier wait gi
 constexpr int kLzMetaSize = 4;
 
 // Planes per streaming stage: the largest divisor K of N/2 with K N^2/4 <=
-// kLzRoleT (one node quad per streaming thread; stages never straddle jx =
+// ST (one node quad per streaming thread; stages never straddle jx =
 // N/2, so the upwind x source is the same cell for the whole stage).  0:
 // unsupported.
-__host__ __device__ constexpr int lz_planes4(int N)
+__host__ __device__ constexpr int lz_planes4(int N, int ST)
 {
     int K = 0;
     for (int k = 1; k <= N / 2; ++k)
-        if ((N / 2) % k == 0 && k * (N * N / 4) <= kLzRoleT) K = k;
+        if ((N / 2) % k == 0 && k * (N * N / 4) <= ST) K = k;
     return K;
+}
+
+// Streaming threads for N nodes per axis: 512 where that raises the busy
+// share by more than 1.4 (above), else 256.
+constexpr int lz_stream_threads(int N)
+{
+    const int q = N * N / 4, s2 = lz_planes4(N, 256) * q, s5 = lz_planes4(N, 512) * q;
+    return 10 * s5 * 256 > 14 * s2 * 512 ? 512 : 256;
 }
 
 // ---------------------------------------------------------------------
@@ -642,9 +660,14 @@ __device__ __forceinline__ void lz_cp16(void *dst, const void *src)
 }
 __device__ __forceinline__ void lz_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void lz_cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void lz_cp_wait_stage()
+// All but the newest n (1 .. kLzMaxStages - 1) groups of this thread's copies
+// have landed.
+__device__ __forceinline__ void lz_cp_wait_but(int n)
 {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kLzStages - 1) : "memory");
+    if (n >= 4) asm volatile("cp.async.wait_group 4;" ::: "memory");
+    else if (n == 3) asm volatile("cp.async.wait_group 3;" ::: "memory");
+    else if (n == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");
 }
 
 // Bulk copies global -> shared through the tensor-memory-access unit
@@ -735,6 +758,7 @@ struct LzArgs {
                             // those copied (a wait that runs out, for tests; normally 0)
     int *fb_count;          // nullable: counts of the fallback's scatter list, zeroed
     int fb_n;               // (fb_n ints) when the step overflowed, before the fallback
+    int stages;             // streaming stages held in shared memory
 };
 
 // Shared memory.  A fixed-layout head (compile-time offsets): warp partial
@@ -743,11 +767,12 @@ struct LzArgs {
 // active node plus a zero entry; the streaming warps fill one while the
 // collision warps use the other), the compact array of collision
 // increments, the per-thread staging slots of the streaming prefetch
-// (kLzStages stages x {own, x source, y source} x streaming threads, 16 bytes
+// (the stages x {own, x source, y source} x streaming threads, 16 bytes
 // each), the active-node bit mask, its word prefixes and the node list.
 struct alignas(128) LzHead {
-    float fpart[3][kLzMaxG][kLzRoleWarps][32];   // warp partials of the F sums, per group (it mod 3)
-    float dpart[2][kLzMaxG][kLzRoleWarps][32];   // warp partials of the D sums, per group (it mod 2)
+    float fpart[kLzMaxG][kLzMaxStreamT / 32][32];    // warp partials of the F sums
+    float ftot[3][kLzMaxG][2][32];               // their totals (sum, error), per group (it mod 3)
+    float dpart[2][kLzMaxG][kLzDParts][32];      // partials of the D sums, per group (it mod 2)
     float4 ta[kLzMaxN];                          // -ax, -ax, A, A
     float4 tv12[kLzMaxN];                        // v, v, v^2, v^2
     float4 tv34[kLzMaxN];                        // v^3, v^3, v^4, v^4
@@ -756,26 +781,27 @@ struct alignas(128) LzHead {
     float2 tcy[kLzMaxG][2][kLzMaxN];             // ca of the cell below (0) and above (1), duplicated
     float mus[kLzMaxG][5][8];                    // mu of own, right, left, below, above (0 outside)
     int4 cell[2][kLzMaxG];                       // c, ix, iy of a group's cells (c < 0: none), per buffer
+    float e0[32];                                // equilibrium sums of the 30 monomials
+    unsigned char px[5][16];                     // lz_psiphi
     int tail_next;                               // next chunk of the increment sums to claim
     int tma_err;                                 // a bounded wait of the bulk-copy ring gave up
-    unsigned long long bar_full[kLzStages];      // bulk-copy ring: stage landed (transaction bytes)
-    unsigned long long bar_empty[kLzStages];     // bulk-copy ring: stage read by the streaming warps
+    unsigned long long bar_full[kLzMaxStages];      // bulk-copy ring: stage landed (transaction bytes)
+    unsigned long long bar_empty[kLzMaxStages];     // bulk-copy ring: stage read by the streaming warps
 };
 constexpr uint32_t kLzAOff = (sizeof(LzHead) + 15) & ~(size_t)15;
 
 struct LzOff {
-    uint32_t abytes, a1, bc, ring, mask, wpre, act, end;
+    uint32_t abytes, a1, bc, ring, mask, act, end;
 };
-__host__ __device__ inline LzOff lz_offsets(int nvt, int mcap, int G)
+__host__ __device__ inline LzOff lz_offsets(int nvt, int mcap, int G, int stages, int S)
 {
     LzOff o;
     o.abytes = (uint32_t)(((sizeof(float) * (size_t)G * (mcap + 1)) + 127) & ~(size_t)127);
     size_t off = kLzAOff + o.abytes;
     o.a1 = (uint32_t)off; off += o.abytes;
     o.bc = (uint32_t)off; off += o.abytes;
-    o.ring = (uint32_t)off; off += (size_t)kLzStages * 3 * kLzRoleT * sizeof(float4);
-    o.mask = (uint32_t)off; off += sizeof(uint32_t) * (nvt / 32);
-    o.wpre = (uint32_t)off; off += sizeof(uint16_t) * (nvt / 32);
+    o.ring = (uint32_t)off; off += (size_t)stages * 3 * S * sizeof(float4);
+    o.mask = (uint32_t)off; off += sizeof(uint2) * (nvt / 32);
     o.act = (uint32_t)off; off += sizeof(uint16_t) * (size_t)mcap;
     o.end = (uint32_t)((off + 15) & ~(size_t)15);
     return o;
@@ -860,35 +886,51 @@ __device__ __forceinline__ float lz_warp_reduce_scatter(float (&v)[32])
     return v[0];
 }
 
-// X (30) from the 26 sums.
-__device__ __forceinline__ void lz_extend(const float *T, float *X)
+// The pivoted fallback of a cell's 5 x 5 solve.
+static __device__ __noinline__ void lz_solve_fallback_p(const Geo *g, const float *P, float *mu)
 {
+    double Pd[19], m8[5];
+    for (int k = 0; k < 19; ++k) Pd[k] = (double)P[k];
+    int f2 = 0;
+    correction_solve<float>(*g, Pd, m8, &f2);
+    for (int k = 0; k < 5; ++k) mu[k] = (float)m8[k];
+}
+__device__ __forceinline__ void lz_solve_fallback(const Geo &g, const float (&P)[19], float (&mu)[5])
+{
+    float p[19], m[5];                 // (copies, so that P and mu stay in registers)
 #pragma unroll
-    for (int k = 0; k < kLzMono; ++k) X[k] = T[k];
-    X[26] = T[4] + T[5] + T[6];
-    X[27] = T[10] + T[15] + T[17];
-    X[28] = T[13] + T[11] + T[18];
-    X[29] = T[14] + T[16] + T[12];
+    for (int k = 0; k < 19; ++k) p[k] = P[k];
+    lz_solve_fallback_p(&g, p, m);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) mu[k] = m[k];
 }
 
-// Correction and output moments of one cell from the sums T (of the
-// post-collision N_c = N + dN) and D (of the collision increment dN): mu to
-// mu_out, moments to mom.  Called by all 32 lanes of a warp (the lanes share
-// the residual of the solve); lane 0 stores.
-__device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, const float *T,
-                                       const float *D, int *fallback)
+// Correction and output moments of one cell from the 26 sums T (of the
+// post-collision N_c = N + dN; the row has room for the 30-entry vector X)
+// and D (of the collision increment dN), both in shared memory: mu to
+// mu_out, moments to mom.  Called by all 32 lanes of a warp: every lane solves
+// the 5 x 5 system (the lanes share its residual), then lane b sums moment b
+// and writes output b.  (With the moments summed by one lane, through arrays
+// in local memory, a solve took 5-8 thousand cycles.)
+__device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, float *T, const float *D,
+                                          const float *e0, const unsigned char (*px)[16], int *fallback)
 {
     const int lane = threadIdx.x & 31;
-    float X[kLzX];
-    lz_extend(T, X);
+    if (lane >= kLzMono && lane < kLzX) {
+        const int i = lane - kLzMono;            // v^2, v_x v^2, v_y v^2, v_z v^2
+        T[lane] = i == 0 ? T[4] + T[5] + T[6] : i == 1 ? T[10] + T[15] + T[17]
+                  : i == 2 ? T[13] + T[11] + T[18] : T[14] + T[16] + T[12];
+    }
+    __syncwarp();
     // Eqs. rinorm_a, correzione: G mu = -D with G from the sums of N_c and
     // D the conserved moments of the increment (1, v, v^2).
     float P[19];
-    for (int k = 0; k < 10; ++k) P[k] = X[k];
-    P[10] = X[27];
-    P[11] = X[28];
-    P[12] = X[29];
-    P[13] = X[20] + X[21] + X[22];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) P[k] = T[k];
+    P[10] = T[27];
+    P[11] = T[28];
+    P[12] = T[29];
+    P[13] = T[20] + T[21] + T[22];
     P[14] = D[0];
     P[15] = D[1];
     P[16] = D[2];
@@ -896,30 +938,42 @@ __device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, 
     P[18] = D[4] + D[5] + D[6];
     float mu[5];
     if (!correction_spd(g, P, mu, lane)) {
-        double Pd[19], m8[5];
-        for (int k = 0; k < 19; ++k) Pd[k] = (double)P[k];
-        int f2 = 0;
-        correction_solve<float>(g, Pd, m8, &f2);
+        lz_solve_fallback(g, P, mu);
         if (lane == 0) ++*fallback;
-        for (int k = 0; k < 5; ++k) mu[k] = (float)m8[k];
     }
-    if (lane != 0) return;
-    float *mo = a.mu_out + (int64_t)c * 8;
-    for (int k = 0; k < 5; ++k) mo[k] = mu[k];
+    if (lane < 5) {
+        float m = mu[0];
+#pragma unroll
+        for (int k = 1; k < 5; ++k) m = lane == k ? mu[k] : m;
+        a.mu_out[(int64_t)c * 8 + lane] = m;
+    }
+    if (!a.mom) return;
     // Moments of h^{n+1}: sum w h phi = sum N_c phi + sum_a mu_a (E0 + eps sum N_c psi_a phi).
     const float eps = g.epsf;
-    float m10[10];
-#pragma unroll
-    for (int b = 0; b < 10; ++b) {
-        float s = X[b];
+    float m = 0.f;
+    if (lane < 10) {
+        m = T[lane];
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-            const int x = lz_psiphi(k, b);
-            s += mu[k] * (a.e0[x] + eps * X[x]);
+            const int x = px[k][lane];
+            m += mu[k] * (e0[x] + eps * T[x]);
         }
-        m10[b] = s;
     }
-    if (a.mom) finalize_moments_f(m10, eps, a.mom + (int64_t)c * 11);
+    // Eqs. densita..sforzi (finalize_moments), output `lane` by lane `lane`.
+    const unsigned all = 0xFFFFFFFFu;
+    const float rho = __shfl_sync(all, m, 0), n = 1.f + eps * rho;
+    const float u0 = __shfl_sync(all, m, 1) / n, u1 = __shfl_sync(all, m, 2) / n, u2 = __shfl_sync(all, m, 3) / n;
+    const float tr = __shfl_sync(all, m, 4) + __shfl_sync(all, m, 5) + __shfl_sync(all, m, 6);
+    const float mq = __shfl_sync(all, m, lane - 1 & 31);
+    const float ua = lane == 5 || lane == 8 || lane == 9 ? u0 : lane == 6 || lane == 10 ? u1 : u2;
+    const float ub = lane == 5 ? u0 : lane == 6 || lane == 8 ? u1 : u2;
+    float o = 2.f * mq - 2.f * eps * n * ua * ub;
+    if (lane == 0) o = rho;
+    if (lane == 1) o = u0;
+    if (lane == 2) o = u1;
+    if (lane == 3) o = u2;
+    if (lane == 4) o = ((2.f / 3.f) * tr - rho) / n - (2.f * eps / 3.f) * (u0 * u0 + u1 * u1 + u2 * u2);
+    if (lane < 11) a.mom[(int64_t)c * 11 + lane] = (double)o;
 }
 
 // The (v_y, v_z) part of a cell's pending correction at a thread's four
@@ -1019,9 +1073,9 @@ struct LzQuad {
     int64_t pbytes;             // bytes per cell (N^3 floats)
     int sbytes;                 // bytes per stage of a cell (S float4)
     uint32_t ring0, ring_end;   // shared addresses: this thread's slots of ring slot 0; ring end
+    uint32_t src;               // bytes between the three sources of a stage (S float4)
+    int stages;
 };
-constexpr uint32_t kLzSrcStride = kLzRoleT * 16;          // between the three sources of a stage
-constexpr uint32_t kLzSlotStride = 3 * kLzSrcStride;      // between stage slots
 
 // Prefetch position of a thread: cell pk of the group, stage pst of that
 // cell, the shared address of the slots it fills next, and what the cell's
@@ -1031,22 +1085,25 @@ struct LzPf {
     int sidx;                // ring slot index of the next stage (bulk-copy ring)
     uint32_t slot;
     const char *own;         // this thread's quad of stage pst of cell pk
-    int64_t yoff;            // byte offset of the y source cell
-    float gxr, gxl;          // ghost values of the right and left walls (cells at a wall)
+    int64_t xoff, yoff;      // byte offsets of the x and y source cells
+    float gx, gxl;           // ghost values of the x source's wall, and of the left one (cells at a wall)
     const float *gy;         // ghost values of the bottom or top wall, by jx (cells at a wall)
-    bool xin_r, xin_l, yin;  // the right, left and y sources are cells
+    bool xin, xin_l, yin;    // the x source (and the left one) and the y source are cells
 };
 
+// v_x < 0 (the first half of the stages): the x source is the right cell;
+// the half ends in lz_prefetch.
 __device__ __forceinline__ void lz_pf_cell(LzPf &p, const LzQuad &q, const Geo &g, const LzArgs &a,
                                            const int4 *cells, const char *hin_t)
 {
     const int4 ce = cells[p.pk];
     p.own = hin_t + (int64_t)ce.x * q.pbytes;
-    p.xin_r = ce.y < g.nx - 1;
+    p.xoff = q.pbytes;
+    p.xin = ce.y < g.nx - 1;
     p.xin_l = ce.y > 0;
     p.yin = q.yup ? ce.z > 0 : ce.z < g.ny - 1;
     p.yoff = q.yup ? -(int64_t)g.nx * q.pbytes : (int64_t)g.nx * q.pbytes;
-    p.gxr = p.xin_r ? 0.f : __ldg(a.ghost + (g.ny + ce.z) * q.N + q.jy);
+    p.gx = p.xin ? 0.f : __ldg(a.ghost + (g.ny + ce.z) * q.N + q.jy);
     p.gxl = p.xin_l ? 0.f : __ldg(a.ghost + ce.z * q.N + q.jy);
     p.gy = a.ghost + (q.yup ? 2 * g.ny + ce.y : 2 * g.ny + g.nx + ce.y) * q.N + q.pl;
 }
@@ -1060,23 +1117,22 @@ __device__ __forceinline__ void lz_prefetch(LzPf &p, const LzQuad &q, const Geo 
     if (q.streams && p.pk < ncell) {
         if (p.pst == 0) lz_pf_cell(p, q, g, a, cells, hin_t);
         lz_cp16s(p.slot, p.own);
-        // x source: the right cell while v_x < 0 (the first half of the
-        // stages), the left cell after.
-        if (p.pst < q.Jh) {
-            if (p.xin_r) lz_cp16s(p.slot + kLzSrcStride, p.own + q.pbytes);
-            else lz_sts4(p.slot + kLzSrcStride, p.gxr);
-        } else {
-            if (p.xin_l) lz_cp16s(p.slot + kLzSrcStride, p.own - q.pbytes);
-            else lz_sts4(p.slot + kLzSrcStride, p.gxl);
-        }
-        if (p.yin) lz_cp16s(p.slot + 2 * kLzSrcStride, p.own + p.yoff);
-        else lz_sts4(p.slot + 2 * kLzSrcStride, __ldg(p.gy + p.pst * q.P4));
+        if (p.xin) lz_cp16s(p.slot + q.src, p.own + p.xoff);
+        else lz_sts4(p.slot + q.src, p.gx);
+        if (p.yin) lz_cp16s(p.slot + 2 * q.src, p.own + p.yoff);
+        else lz_sts4(p.slot + 2 * q.src, __ldg(p.gy + p.pst * q.P4));
         p.own += q.sbytes;
     }
     lz_cp_commit();
-    p.slot += kLzSlotStride;
+    p.slot += 3 * q.src;
     if (p.slot == q.ring_end) p.slot = q.ring0;
-    if (++p.pst == q.J) {
+    ++p.pst;
+    if (p.pst == q.Jh) {                         // v_x > 0 from here on: the left cell
+        p.xoff = -q.pbytes;
+        p.xin = p.xin_l;
+        p.gx = p.gxl;
+    }
+    if (p.pst == q.J) {
         p.pst = 0;
         ++p.pk;
     }
@@ -1105,11 +1161,10 @@ __device__ __forceinline__ void lz_prefetch_tma(LzPf &p, const LzQuad &q, const 
 {
     if (p.pk < ncell) {
         if (p.pst == 0) lz_pf_cell(p, q, g, a, cells, hin_t);
-        const bool left = p.pst >= q.Jh;
-        const bool xin = left ? p.xin_l : p.xin_r;
+        const bool left = p.pst >= q.Jh, xin = p.xin;
         if (q.streams) {
-            if (!xin) lz_sts4(p.slot + kLzSrcStride, left ? p.gxl : p.gxr);
-            if (!p.yin) lz_sts4(p.slot + 2 * kLzSrcStride, __ldg(p.gy + p.pst * q.P4));
+            if (!xin) lz_sts4(p.slot + q.src, p.gx);
+            if (!p.yin) lz_sts4(p.slot + 2 * q.src, __ldg(p.gy + p.pst * q.P4));
         }
         // After a wait gave up, nothing more is issued (the waits are skipped).
         if (threadIdx.x == 0 && *(volatile int *)&H.tma_err == 0) {
@@ -1129,22 +1184,28 @@ __device__ __forceinline__ void lz_prefetch_tma(LzPf &p, const LzQuad &q, const 
             const uint32_t ybytes = (uint32_t)q.P4 * hb * ((above ? 1u : 0u) + (below ? 1u : 0u));
             lz_mbar_expect_tx(full, sb * (1u + (xin ? 1u : 0u)) + ybytes + extra);
             lz_bulk_g2s(p.slot, p.own, sb, full);
-            if (xin) lz_bulk_g2s(p.slot + kLzSrcStride, left ? p.own - q.pbytes : p.own + q.pbytes, sb, full);
+            if (xin) lz_bulk_g2s(p.slot + q.src, left ? p.own - q.pbytes : p.own + q.pbytes, sb, full);
             const int64_t ystep = (int64_t)g.nx * q.pbytes;
             for (int pl = 0; pl < q.P4; ++pl) {
                 const uint32_t o = (uint32_t)pl * 2u * hb;
-                if (above) lz_bulk_g2s(p.slot + 2 * kLzSrcStride + o, p.own + ystep + o, hb, full);
-                if (below) lz_bulk_g2s(p.slot + 2 * kLzSrcStride + o + hb, p.own - ystep + o + hb, hb, full);
+                if (above) lz_bulk_g2s(p.slot + 2 * q.src + o, p.own + ystep + o, hb, full);
+                if (below) lz_bulk_g2s(p.slot + 2 * q.src + o + hb, p.own - ystep + o + hb, hb, full);
             }
         }
         p.own += q.sbytes;
     }
-    p.slot += kLzSlotStride;
-    if (++p.sidx == kLzStages) {
+    p.slot += (3 * q.src);
+    if (++p.sidx == q.stages) {
         p.sidx = 0;
         p.slot = q.ring0;
     }
-    if (++p.pst == q.J) {
+    ++p.pst;
+    if (p.pst == q.Jh) {
+        p.xoff = -q.pbytes;
+        p.xin = p.xin_l;
+        p.gx = p.gxl;
+    }
+    if (p.pst == q.J) {
         p.pst = 0;
         ++p.pk;
     }
@@ -1163,12 +1224,12 @@ struct LzAcc {
 // active nodes of the quad to the compact array (component k of G).  SX:
 // stretched cells, the x Courant numbers times the cell's factor fx2.
 template <int G, bool SX>
-__device__ __forceinline__ void lz_stream_stage(uint32_t sl, int jx, int j0, int k, const LzHead &H,
+__device__ __forceinline__ void lz_stream_stage(uint32_t sl, uint32_t src, int jx, int j0, int k, const LzHead &H,
                                                 const float4 *tcx, const float2 *tcy, LzAcc &c,
-                                                float4 *dst, const uint32_t *smask, const uint16_t *swpre,
-                                                float *Af, float2 eps2, float2 one2, float2 nay2, float2 fx2)
+                                                float4 *dst, const uint2 *smask, float *Af,
+                                                float2 eps2, float2 one2, float2 nay2, float2 fx2)
 {
-    const float4 h0 = lz_lds4(sl), hx = lz_lds4(sl + kLzSrcStride), hy = lz_lds4(sl + 2 * kLzSrcStride);
+    const float4 h0 = lz_lds4(sl), hx = lz_lds4(sl + src), hy = lz_lds4(sl + 2 * src);
     const float4 cx4 = tcx[jx];
     const float2 cy2 = tcy[jx];
     const float4 ta = H.ta[jx];
@@ -1177,6 +1238,7 @@ __device__ __forceinline__ void lz_stream_stage(uint32_t sl, int jx, int j0, int
     const float2 h0p[2] = {lz_lo(h0), lz_hi(h0)}, hxp[2] = {lz_lo(hx), lz_hi(hx)},
                  hyp[2] = {lz_lo(hy), lz_hi(hy)};
     float2 ht[2];
+    const float2 mone2 = lz_dup(-1.f);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         // u = h_c + (1 + eps h_c) kappa of each source, as h_c (1 + eps kappa) + kappa.
@@ -1187,9 +1249,8 @@ __device__ __forceinline__ void lz_stream_stage(uint32_t sl, int jx, int j0, int
         const float2 ky = lz_add2(cy2, c.bdy[p]);
         const float2 uy = lz_fma2(hyp[p], lz_fma2(eps2, ky, one2), ky);
         // Eq. streaming2D: u0 - ax (u0 - ux) - ay (u0 - uy).
-        const float2 mux = make_float2(-ux.x, -ux.y), muy = make_float2(-uy.x, -uy.y);
-        float2 h = lz_fma2(nax2, lz_add2(u0, mux), u0);
-        h = lz_fma2(nay2, lz_add2(u0, muy), h);
+        float2 h = lz_fma2(nax2, lz_fma2(ux, mone2, u0), u0);
+        h = lz_fma2(nay2, lz_fma2(uy, mone2, u0), h);
         ht[p] = h;
         const float2 n = lz_mul2(h, A2);
         c.s0[p] = lz_add2(c.s0[p], n);
@@ -1200,11 +1261,11 @@ __device__ __forceinline__ void lz_stream_stage(uint32_t sl, int jx, int j0, int
     }
     *dst = make_float4(ht[0].x, ht[0].y, ht[1].x, ht[1].y);
     // Active nodes of the quad (nodes j0 .. j0 + 3) go to the compact array.
-    const uint32_t mw = smask[j0 >> 5];
+    const uint2 mw = smask[j0 >> 5];
     const int sh = j0 & 31;
-    const uint32_t bits = (mw >> sh) & 15u;
+    const uint32_t bits = (mw.x >> sh) & 15u;
     if (bits) {
-        int mi = swpre[j0 >> 5] + __popc(mw & ((1u << sh) - 1u));
+        int mi = (int)mw.y + __popc(mw.x & ((1u << sh) - 1u));
         const float hv[4] = {ht[0].x, ht[0].y, ht[1].x, ht[1].y};
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -1228,25 +1289,35 @@ __device__ __forceinline__ void lz_term(float4 ha, float4 hb, float2 eps2, float
     acc = make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// The state of a thread's run: the sum of its current destination, which is
-// stored when the destination's last term has passed (atomically for the
-// thread's first destination and its unfinished last one, which neighbouring
-// runs may share).
+// The state of a thread's run: the sum of its current destination and the
+// shared addresses where that and the next destination's go.  A destination
+// ends with one predicated store.  (With an atomic branch for the first
+// destination in each of the 24 unrolled terms, the terms of four cells took
+// 104 thousand cycles at 32^3 and 2x10^4 samples instead of 61.)  Neighbouring
+// runs may share a thread's first destination and its unfinished last one, so
+// the first sum goes to a slot of the thread's own (at first p is the slot);
+// both are added to the increments atomically at the end of the run.
 template <typename V> struct LzRun {
     V acc;
-    int dest;
-    bool first;
+    uint32_t p, next;
 };
+__device__ __forceinline__ void lz_sts(uint32_t dst, float4 v)
+{
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void lz_sts(uint32_t dst, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(v.x), "f"(v.y) : "memory");
+}
 
 template <typename V>
-__device__ __forceinline__ void lz_apply(V ha, V hb, uint2 r, float2 eps2, LzRun<V> &st, V *Bv)
+__device__ __forceinline__ void lz_apply(V ha, V hb, uint2 r, float2 eps2, LzRun<V> &st)
 {
     lz_term(ha, hb, eps2, lz_dup(__uint_as_float(r.y)), st.acc);
-    if (r.x & 1u) {
-        if (st.first) lz_atomic_add(Bv + st.dest, st.acc);
-        else Bv[st.dest] = st.acc;
-        st.first = false;
-        ++st.dest;
+    if (r.x & 1u) {                              // the destination's last term
+        lz_sts(st.p, st.acc);
+        st.p = st.next;
+        st.next += sizeof(V);
         lz_set_zero(st.acc);
     }
 }
@@ -1254,8 +1325,7 @@ __device__ __forceinline__ void lz_apply(V ha, V hb, uint2 r, float2 eps2, LzRun
 // Applies 8 records (the operands of two terms are read before either of
 // them can store a destination's sum).
 template <typename V, uint32_t AMASK>
-__device__ __forceinline__ void lz_apply8(const uint2 (&r)[8], const char *Ab, float2 eps2, LzRun<V> &st,
-                                          V *Bv)
+__device__ __forceinline__ void lz_apply8(const uint2 (&r)[8], const char *Ab, float2 eps2, LzRun<V> &st)
 {
 #pragma unroll
     for (int h = 0; h < 8; h += 2) {
@@ -1263,26 +1333,27 @@ __device__ __forceinline__ void lz_apply8(const uint2 (&r)[8], const char *Ab, f
         const V hb0 = *reinterpret_cast<const V *>(Ab + (r[h].x >> 16));
         const V ha1 = *reinterpret_cast<const V *>(Ab + (r[h + 1].x & AMASK));
         const V hb1 = *reinterpret_cast<const V *>(Ab + (r[h + 1].x >> 16));
-        lz_apply(ha0, hb0, r[h], eps2, st, Bv);
-        lz_apply(ha1, hb1, r[h + 1], eps2, st, Bv);
+        lz_apply(ha0, hb0, r[h], eps2, st);
+        lz_apply(ha1, hb1, r[h + 1], eps2, st);
     }
 }
 
-// Barrier among the 256 threads of one role (named barrier 1: streaming,
-// 2: collision; 0 is __syncthreads).
-__device__ __forceinline__ void lz_role_bar(int id)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kLzRoleT) : "memory");
-}
+// Barriers among the threads of one role (named barrier 1: streaming, 2:
+// collision; 0 is __syncthreads).
+template <int ST>
+__device__ __forceinline__ void lz_stream_bar() { asm volatile("bar.sync 1, %0;" ::"n"(ST) : "memory"); }
+__device__ __forceinline__ void lz_coll_bar() { asm volatile("bar.sync 2, %0;" ::"n"(kLzCollT) : "memory"); }
 // Named barrier 3 over all threads: the collision role arrives without
 // waiting once its terms are complete; the streaming role waits for that.
+template <int ST>
 __device__ __forceinline__ void lz_terms_done_arrive()
 {
-    asm volatile("bar.arrive 3, %0;" ::"n"(kLzThreads) : "memory");
+    asm volatile("bar.arrive 3, %0;" ::"n"(lz_threads(ST)) : "memory");
 }
+template <int ST>
 __device__ __forceinline__ void lz_terms_done_wait()
 {
-    asm volatile("bar.sync 3, %0;" ::"n"(kLzThreads) : "memory");
+    asm volatile("bar.sync 3, %0;" ::"n"(lz_threads(ST)) : "memory");
 }
 constexpr int kLzTailChunk = 256;  // active nodes per claimed chunk of the increment sums
 
@@ -1301,17 +1372,18 @@ constexpr int kLzTailChunk = 256;  // active nodes per claimed chunk of the incr
 // every stage; a stage covers K planes and a cell J = N / K stages.
 //
 // TMA: the streaming sources arrive by bulk copies (cp.async.bulk) that
-// thread 0 of the role issues into a ring of kLzStages slots, with a full
+// thread 0 of the role issues into a ring of slots, with a full
 // and an empty mbarrier per slot, instead of per-thread cp.async.
 //
 // lz_run runs the pipeline of one CTA over the groups grp0, grp0 + gstride,
 // ... (nmine of them) of one problem; the kernel k_lz gives CTA b the groups
 // b, b + gridDim.x, ...
-template <int G, int NV, bool SX, bool TMA = false>
+template <int G, int NV, bool SX, int ST, bool TMA = false>
 __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem_raw, int grp0, int gstride,
                                        int nmine)
 {
     using V = typename LzVec<G>::T;
+    constexpr int kThreads = lz_threads(ST), kStreamWarps = ST / 32;
     if (a.meta[1]) {                              // too many active nodes: k_cell4 runs
         if (a.fb_count)
             for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < a.fb_n; i += gridDim.x * blockDim.x)
@@ -1320,26 +1392,25 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
     }
     const int N = NV ? NV : g.nv;
     const int N2 = N * N, nvt = N2 * N, t = threadIdx.x;
-    const int Qd = N2 / 4, nq = N / 4, P4 = lz_planes4(N), J = N / P4, Jh = J / 2;
+    const int Qd = N2 / 4, nq = N / 4, P4 = lz_planes4(N, ST), J = N / P4, Jh = J / 2;
     const int S = P4 * Qd;                        // float4 per stage (the threads that stream)
     const int half = N / 2;
     const int64_t plane4 = nvt / 4;               // float4 per cell
     LzHead &H = *reinterpret_cast<LzHead *>(smem_raw);
     const int M = a.meta[0];
-    const LzOff so = lz_offsets(nvt, a.mcap, G);
+    const LzOff so = lz_offsets(nvt, a.mcap, G, a.stages, S);
     float4 *ring = reinterpret_cast<float4 *>(smem_raw + so.ring);
     V *Bv = reinterpret_cast<V *>(smem_raw + so.bc);
     float *Bf = reinterpret_cast<float *>(smem_raw + so.bc);
-    uint32_t *smask = reinterpret_cast<uint32_t *>(smem_raw + so.mask);
-    uint16_t *swpre = reinterpret_cast<uint16_t *>(smem_raw + so.wpre);
+    uint2 *smask = reinterpret_cast<uint2 *>(smem_raw + so.mask);   // mask word, compact index of its first node
     uint16_t *sact = reinterpret_cast<uint16_t *>(smem_raw + so.act);
     const float eps = g.epsf;
     const float2 eps2 = lz_dup(eps), one2 = lz_dup(1.f);
     const int lane = t & 31, warp = t >> 5;
-    const bool streamer = t < kLzRoleT;
+    const bool streamer = t < ST;
 
     // ---- tables (once per launch) ----------------------------------------
-    for (int i = t; i < N; i += kLzThreads) {
+    for (int i = t; i < N; i += kThreads) {
         const double v = g.axv[i], A = g.axA[i];
         // Courant numbers 0 without streaming: h~ is then exactly the
         // corrected input (every source term is multiplied by zero).
@@ -1353,16 +1424,20 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
         H.tv12[i] = make_float4(fv, fv, v2, v2);
         H.tv34[i] = make_float4(v3, v3, v4, v4);
     }
-    for (int w = t; w < nvt / 32; w += kLzThreads) {
-        smask[w] = a.mask[w];
-        swpre[w] = (uint16_t)a.wpre[w];
+    for (int w = t; w < nvt / 32; w += kThreads) {
+        smask[w] = make_uint2(a.mask[w], (uint32_t)a.wpre[w]);
     }
-    for (int m = t; m < M; m += kLzThreads) sact[m] = (uint16_t)a.act[m];
-    for (int i = t; i < 2 * kLzMaxG * kLzRoleWarps * 32; i += kLzThreads) (&H.dpart[0][0][0][0])[i] = 0.f;
+    for (int m = t; m < M; m += kThreads) {     // active nodes as jx << 10 | jy << 5 | jz
+        const int j = a.act[m], jxy = j / N, jx = jxy / N;
+        sact[m] = (uint16_t)(jx << 10 | (jxy - jx * N) << 5 | (j - jxy * N));
+    }
+    for (int i = t; i < 2 * kLzMaxG * kLzDParts * 32; i += kThreads) (&H.dpart[0][0][0][0])[i] = 0.f;
+    if (t < kLzX) H.e0[t] = a.e0[t];
+    if (t < 50) H.px[t / 10][t % 10] = (unsigned char)lz_psiphi(t / 10, t % 10);
     if (TMA && t == 0) {
-        for (int s = 0; s < kLzStages; ++s) {
+        for (int s = 0; s < a.stages; ++s) {
             lz_mbar_init(lz_saddr(&H.bar_full[s]), 1);
-            lz_mbar_init(lz_saddr(&H.bar_empty[s]), kLzRoleWarps);
+            lz_mbar_init(lz_saddr(&H.bar_empty[s]), kStreamWarps);
         }
         H.tma_err = 0;
         lz_mbar_init_fence();
@@ -1381,6 +1456,35 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
     LzTmaProd prod{0u, 0u, 0u};                   // thread 0: the bulk-copy ring's producer state
     uint32_t fpar = 0u;                           // parity of each slot's next full phase
 
+    // One warp per cell of group it - 2: totals over the warps, then the
+    // correction and the moments (k: the warp's number within its role).
+    auto solve = [&](int it, int k) {
+        if (it < 2) return;
+        const int grp = grp0 + (it - 2) * gstride, fb = (it - 2) % 3, db = it & 1, kc = grp * G + k;
+        if (k >= G || kc >= g.nr) return;
+        if (lane < kLzMono) {
+            // Compensated totals over the warps: T = F + D (the sums of N_c)
+            // and D.
+            const float f = H.ftot[fb][k][0][lane], fc = H.ftot[fb][k][1][lane];
+            float d = 0.f, dc = 0.f;
+#pragma unroll
+            for (int w = 0; w < kLzDParts; ++w) {
+                float e;
+                two_sum(d, H.dpart[db][k][w][lane], d, e);
+                dc = __fadd_rn(dc, e);
+            }
+            float tt, te;
+            two_sum(f, d, tt, te);
+            H.ftot[fb][k][0][lane] = __fadd_rn(tt, __fadd_rn(te, __fadd_rn(fc, dc)));
+            H.dpart[db][k][0][lane] = __fadd_rn(d, dc);
+        }
+        __syncwarp();
+        lz_finish(g, a, cell_of(g, kc), H.ftot[fb][k][0], H.dpart[db][k][0], H.e0, H.px, &fallback);
+        __syncwarp();
+        // The slots take the increment sums of a later group (atomically).
+        for (int i = lane; i < kLzDParts * 32; i += 32) (&H.dpart[db][k][0][0])[i] = 0.f;
+    };
+
     // Iteration it: the streaming warps take this CTA's group it, the
     // collision warps its group it - 1.
     for (int it = 0; it <= nmine + 1; ++it) {
@@ -1395,12 +1499,12 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     const int c = kc < g.nr ? cell_of(g, kc) : -1;
                     H.cell[buf][t] = make_int4(c, c >= 0 ? c % g.nx : 0, c >= 0 ? c / g.nx : 0, 0);
                 }
-                lz_role_bar(1);
+                lz_stream_bar<ST>();
                 int ncell = 0;
 #pragma unroll
                 for (int k = 0; k < G; ++k) ncell += H.cell[buf][k].x >= 0 ? 1 : 0;
                 // mu of the five cells each cell's streaming reads (0 outside the cavity).
-                for (int i = t; i < G * 40; i += kLzRoleT) {
+                for (int i = t; i < G * 40; i += ST) {
                     const int k = i / 40, r = i - k * 40, s5 = r / 8, m = r - s5 * 8;
                     const int4 ce = H.cell[buf][k];
                     int cs = ce.x;
@@ -1411,24 +1515,24 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     if (s5 == 4) { ok = ok && ce.z < g.ny - 1; cs = ce.x + g.nx; }
                     H.mus[k][s5][m] = ok ? a.mu_in[(int64_t)cs * 8 + m] : 0.f;
                 }
-                // kLzStages - 1 stages in flight ahead of the one being used.
+                // a.stages - 1 stages in flight ahead of the one being used.
                 const uint32_t ring0 = lz_saddr(ring) + t * 16;
                 const LzQuad qd{S, J, Jh, P4, pl, N, jy, yup, streams, (int64_t)nvt * 4, S * 16, ring0,
-                                ring0 + kLzStages * kLzSlotStride};
+                                ring0 + a.stages * 3 * S * 16, (uint32_t)(S * 16), a.stages};
                 const char *hin_t = reinterpret_cast<const char *>(hin4 + t);
                 LzPf pf{};
                 pf.slot = ring0;
                 const int4 *cells = H.cell[buf];
-#pragma unroll
-                for (int kk = 0; kk < kLzStages - 1; ++kk) {
+#pragma unroll 1
+                for (int kk = 0; kk < a.stages - 1; ++kk) {
                     if (TMA) lz_prefetch_tma(pf, qd, g, a, cells, hin_t, ncell, H, prod);
                     else lz_prefetch(pf, qd, g, a, cells, hin_t, ncell);
                 }
-                lz_role_bar(1);
+                lz_stream_bar<ST>();
                 // Correction tables of the group's cells: ca(jx) = mu_0 + mu_x
                 // v_x + mu_4 v_x^2 of the own cell, the upwind x cell (right for
                 // jx < N/2, left otherwise), and the cells below and above.
-                for (int i = t; i < G * N; i += kLzRoleT) {
+                for (int i = t; i < G * N; i += ST) {
                     const int k = i / N, jx = i - k * N;
                     const float vx = H.v[jx];
                     float ca[5];
@@ -1442,7 +1546,7 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     H.tcy[k][0][jx] = lz_dup(ca[3]);
                     H.tcy[k][1][jx] = lz_dup(ca[4]);
                 }
-                lz_role_bar(1);
+                lz_stream_bar<ST>();
 
                 // ---- streaming with the deferred correction applied to its sources
                 uint32_t cslot = ring0;           // slots of the stage being used
@@ -1473,7 +1577,7 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
 #pragma unroll 1
                     for (int st = 0; st < J; ++st) {
                         if (st == Jh) lz_bd(H.mus[k][2], H.v, jy, qz, ac.bdx);   // the left cell now
-                        // The slots read last stage take the stage kLzStages - 1
+                        // The slots read last stage take the stage a.stages - 1
                         // ahead; then this stage's copies have landed.
                         if (TMA) {
                             lz_prefetch_tma(pf, qd, g, a, cells, hin_t, ncell, H, prod);
@@ -1481,10 +1585,10 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                             fpar ^= 1u << cidx;
                         } else {
                             lz_prefetch(pf, qd, g, a, cells, hin_t, ncell);
-                            lz_cp_wait_stage();
+                            lz_cp_wait_but(a.stages - 1);
                         }
                         if (streams)
-                            lz_stream_stage<G, SX>(cslot, jx, j0, k, H, tcx, tcy, ac, dst, smask, swpre, Af,
+                            lz_stream_stage<G, SX>(cslot, qd.src, jx, j0, k, H, tcx, tcy, ac, dst, smask, Af,
                                                    eps2, one2, nay2k, fx2);
                         if (TMA) {
                             // The warp has read the slot: release it to the producer.
@@ -1492,9 +1596,9 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                             __syncwarp();
                             if (lane == 0) lz_mbar_arrive(lz_saddr(&H.bar_empty[cidx]));
                         }
-                        cslot += kLzSlotStride;
+                        cslot += 3 * qd.src;
                         if (TMA) {
-                            if (++cidx == kLzStages) {
+                            if (++cidx == a.stages) {
                                 cidx = 0;
                                 cslot = ring0;
                             }
@@ -1525,44 +1629,30 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                             lz_mono_from_powers(si, H.v[jy], H.v[4 * qz + i], Msum);
                         }
                     }
-                    H.fpart[it % 3][k][warp][lane] = lz_warp_reduce_scatter(Msum);
+                    H.fpart[k][warp][lane] = lz_warp_reduce_scatter(Msum);
                 }
                 if (!TMA) lz_cp_wait_all();
-            }
-            if (clk && t == 0) a.clk[it * kClkPhases + 1] = clock64();
-            // One warp per cell of group it - 2: totals over the warps, then the
-            // correction and the moments.
-            if (it >= 2) {
-                const int grp = grp0 + (it - 2) * gstride, fb = (it - 2) % 3, db = it & 1;
-                const int k = warp, kc = grp * G + k;
-                if (k < G && kc < g.nr) {
-                    if (lane < kLzMono) {
-                        // Compensated totals over the warps: T = F + D (the
-                        // sums of N_c) and D.
-                        float f = 0.f, fc = 0.f, d = 0.f, dc = 0.f;
+                // Compensated totals over the warps, one warp per cell.
+                lz_stream_bar<ST>();
+                if (warp < G && lane < kLzMono) {
+                    float f = 0.f, fc = 0.f;
 #pragma unroll
-                        for (int w = 0; w < kLzRoleWarps; ++w) {
-                            float e;
-                            two_sum(f, H.fpart[fb][k][w][lane], f, e);
-                            fc = __fadd_rn(fc, e);
-                            two_sum(d, H.dpart[db][k][w][lane], d, e);
-                            dc = __fadd_rn(dc, e);
-                        }
-                        float tt, te;
-                        two_sum(f, d, tt, te);
-                        H.fpart[fb][k][0][lane] = __fadd_rn(tt, __fadd_rn(te, __fadd_rn(fc, dc)));
-                        H.dpart[db][k][0][lane] = __fadd_rn(d, dc);
+                    for (int w = 0; w < kStreamWarps; ++w) {
+                        float e;
+                        two_sum(f, H.fpart[warp][w][lane], f, e);
+                        fc = __fadd_rn(fc, e);
                     }
-                    __syncwarp();
-                    lz_finish(g, a, cell_of(g, kc), H.fpart[fb][k][0], H.dpart[db][k][0], &fallback);
-                    __syncwarp();
-                    // The slots take the increment sums of a later group (atomically).
-                    for (int i = lane; i < kLzRoleWarps * 32; i += 32) (&H.dpart[db][k][0][0])[i] = 0.f;
+                    H.ftot[it % 3][warp][0][lane] = f;
+                    H.ftot[it % 3][warp][1][lane] = fc;
                 }
             }
+            if (clk && t == 0) a.clk[it * kClkPhases + 1] = clock64();
             if (clk && t == 0) a.clk[it * kClkPhases + 5] = clock64();
-        } else if (it >= 1 && it <= nmine) {
-            const int tc = t - kLzRoleT, buf = (it - 1) & 1;
+        } else {
+            solve(it, warp - kStreamWarps);
+        }
+        if (!streamer && it >= 1 && it <= nmine) {
+            const int tc = t - ST, buf = (it - 1) & 1;
             char *Ab = smem_raw + kLzAOff + buf * so.abytes;
             float *Af = reinterpret_cast<float *>(Ab);
             int ncell = 0, cg[G];
@@ -1574,32 +1664,35 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
             // ---- Monte Carlo terms (Eq. monteCarloInt) ----------------------
             // The increments start from zero; the zero entry M of h~ stands for
             // nodes outside the grid, and cells missing from a short group hold 0.
-            for (int i = tc; i < M + 1; i += kLzRoleT) lz_set_zero(Bv[i]);
+            for (int i = tc; i < M + 1; i += kLzCollT) lz_set_zero(Bv[i]);
             if (tc < G) Af[M * G + tc] = 0.f;
             if (tc == 0) H.tail_next = 0;
             if (ncell < G)
-                for (int i = tc; i < M * G; i += kLzRoleT)
+                for (int i = tc; i < M * G; i += kLzCollT)
                     if (i % G >= ncell) Af[i] = 0.f;
-            lz_role_bar(2);
+            lz_coll_bar();
             {
                 // Each thread applies its run of the destination-sorted terms:
                 // it sums one destination's terms in registers and stores the
-                // sum when the destination's last term has passed (atomically
-                // for its first destination and its unfinished last one, which
-                // neighbouring runs may share).
+                // sum when the destination's last term has passed (LzRun).
                 const int C = a.meta[3];
                 if (C > 0) {
                     constexpr uint32_t amask = G == 4 ? 0xFFF0u : 0xFFF8u;
                     LzRun<V> st;
+                    // The slot: 16 bytes of the increment sums' slots, idle
+                    // (zero) until the terms are done.
+                    V *const first = reinterpret_cast<V *>(&H.dpart[buf][0][0][0] + 4 * tc);
+                    const int dest0 = a.dest0[tc];
+                    const uint32_t slot = lz_saddr(first);
                     lz_set_zero(st.acc);
-                    st.dest = a.dest0[tc];
-                    st.first = true;
+                    st.p = slot;
+                    st.next = lz_saddr(Bv + dest0 + 1);
                     // Batches of 8 records in three register buffers: a buffer
                     // is refilled as soon as it has been applied, two batches
                     // ahead (the records stream from L2).  A run is C records,
                     // C a multiple of 8, zero-padded by the plan.
                     const uint2 *rp = a.rec + tc;
-                    constexpr int Ts = kLzRoleT, Bs = 8 * kLzRoleT;
+                    constexpr int Ts = kLzCollT, Bs = 8 * kLzCollT;
                     uint2 r0[8], r1[8], r2[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
@@ -1609,47 +1702,51 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     }
                     for (int i = 0; i < C; i += 24) {
                         rp += 3 * Bs;
-                        lz_apply8<V, amask>(r0, Ab, eps2, st, Bv);
+                        lz_apply8<V, amask>(r0, Ab, eps2, st);
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
                             if (i + 24 < C) r0[u] = rp[u * Ts];
                         if (i + 8 < C) {
-                            lz_apply8<V, amask>(r1, Ab, eps2, st, Bv);
+                            lz_apply8<V, amask>(r1, Ab, eps2, st);
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (i + 32 < C) r1[u] = rp[Bs + u * Ts];
                         }
                         if (i + 16 < C) {
-                            lz_apply8<V, amask>(r2, Ab, eps2, st, Bv);
+                            lz_apply8<V, amask>(r2, Ab, eps2, st);
 #pragma unroll
                             for (int u = 0; u < 8; ++u)
                                 if (i + 40 < C) r2[u] = rp[2 * Bs + u * Ts];
                         }
                     }
-                    lz_atomic_add(Bv + st.dest, st.acc);
+                    const bool ended = st.p != slot;      // the first destination's sum is in the slot
+                    lz_atomic_add(ended ? Bv + (st.p - lz_saddr(Bv)) / sizeof(V) : Bv + dest0, st.acc);
+                    if (ended) {
+                        lz_atomic_add(Bv + dest0, *first);
+                        lz_set_zero(*first);
+                    }
                 }
             }
             if (clk && tc == 0) a.clk[it * kClkPhases + 2] = clock64();
-            if (NV != 32 && a.early_tail) {
+            if (a.early_tail) {
                 // The increments are complete once every collision thread is here.
-                lz_role_bar(2);
-                lz_terms_done_arrive();
+                lz_coll_bar();
+                lz_terms_done_arrive<ST>();
             }
         }
         // ---- sums of the collision increment and h_c = h~ + dN / w on the
         // active nodes of group it - 1, two cells at a time.  Either all
         // warps after a CTA barrier, each with a fixed share of the nodes and
         // its partial sums added to the slots of warp (warp mod 8); or
-        // (early tail, for when the collision terms take less time than the
-        // streaming; never at 32^3 velocities) the collision warps as soon as
-        // their terms are complete and the streaming warps once they are
+        // (early tail, the default: the collision terms take less time than the
+        // streaming) the collision warps as soon as their terms are complete and the streaming warps once they are
         // done, every warp claiming chunks of kLzTailChunk nodes of one cell
         // pair at a time (pair 0 first) and adding its partial sums of a pair
         // to the slots when it moves on.
         if (it >= 1 && it <= nmine) {
-            const bool early = NV != 32 && a.early_tail;
+            const bool early = a.early_tail;
             if (early) {
-                if (streamer) lz_terms_done_wait();
+                if (streamer) lz_terms_done_wait<ST>();
             } else {
                 __syncthreads();
             }
@@ -1662,16 +1759,16 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                 ncell += cg[k] >= 0 ? 1 : 0;
             }
             if (!early) {
-                const int u = t ^ kLzRoleT;
+                const int u = streamer ? t + kLzCollT : t - ST;
 #pragma unroll
                 for (int k2 = 0; k2 < G; k2 += 2) {
                     float2 D2[32];
 #pragma unroll
                     for (int r = 0; r < 32; ++r) D2[r] = lz_zero2();
                     if (k2 < ncell) {
-                        for (int mm = u; mm < M; mm += kLzThreads) {
-                            const int j = sact[mm], jxy = j / N;
-                            const int jx = jxy / N, jyy = jxy - jx * N, jz = j - jxy * N;
+                        for (int mm = u; mm < M; mm += kThreads) {
+                            const int pk = sact[mm], jx = pk >> 10, jyy = pk >> 5 & 31, jz = pk & 31;
+                            const int j = (jx * N + jyy) * N + jz;
                             const float2 d = *reinterpret_cast<const float2 *>(Bf + mm * G + k2);
                             const float2 h = *reinterpret_cast<const float2 *>(Af + mm * G + k2);
                             const float x = H.v[jx], x2 = x * x;
@@ -1684,8 +1781,8 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                         }
                     }
                     const float2 r = lz_warp_reduce_scatter2(D2);
-                    atomicAdd(&H.dpart[buf][k2][warp & (kLzRoleWarps - 1)][lane], r.x);
-                    atomicAdd(&H.dpart[buf][k2 + 1][warp & (kLzRoleWarps - 1)][lane], r.y);
+                    atomicAdd(&H.dpart[buf][k2][warp & (kLzDParts - 1)][lane], r.x);
+                    atomicAdd(&H.dpart[buf][k2 + 1][warp & (kLzDParts - 1)][lane], r.y);
                 }
             } else {
                 const int npair = (ncell + 1) / 2, per = (M + kLzTailChunk - 1) / kLzTailChunk;
@@ -1702,8 +1799,8 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     if (k2 != kcur) {
                         if (kcur >= 0) {
                             const float2 r = lz_warp_reduce_scatter2(D2);
-                            atomicAdd(&H.dpart[buf][kcur][warp & (kLzRoleWarps - 1)][lane], r.x);
-                            atomicAdd(&H.dpart[buf][kcur + 1][warp & (kLzRoleWarps - 1)][lane], r.y);
+                            atomicAdd(&H.dpart[buf][kcur][warp & (kLzDParts - 1)][lane], r.x);
+                            atomicAdd(&H.dpart[buf][kcur + 1][warp & (kLzDParts - 1)][lane], r.y);
 #pragma unroll
                             for (int r2 = 0; r2 < 32; ++r2) D2[r2] = lz_zero2();
                         }
@@ -1712,8 +1809,8 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     if (k2 < 0) break;
                     const int m0 = (ch - (k2 / 2) * per) * kLzTailChunk, m1 = min(M, m0 + kLzTailChunk);
                     for (int mm = m0 + lane; mm < m1; mm += 32) {
-                        const int j = sact[mm], jxy = j / N;
-                        const int jx = jxy / N, jyy = jxy - jx * N, jz = j - jxy * N;
+                        const int pk = sact[mm], jx = pk >> 10, jyy = pk >> 5 & 31, jz = pk & 31;
+                        const int j = (jx * N + jyy) * N + jz;
                         const float2 d = *reinterpret_cast<const float2 *>(Bf + mm * G + k2);
                         const float2 h = *reinterpret_cast<const float2 *>(Af + mm * G + k2);
                         const float x = H.v[jx], x2 = x * x;
@@ -1726,8 +1823,8 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     }
                 }
             }
-            if (clk && t == kLzRoleT) a.clk[it * kClkPhases + 3] = clock64();
-            if (clk && t == kLzRoleT) a.clk[it * kClkPhases + 4] = clock64();
+            if (clk && t == ST) a.clk[it * kClkPhases + 3] = clock64();
+            if (clk && t == ST) a.clk[it * kClkPhases + 4] = clock64();
         }
         __syncthreads();
     }
@@ -1737,18 +1834,18 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
         // issued into each slot before the CTA leaves (after the first
         // timeout nothing more was issued).
         if (a.err) atomicOr(a.err, 1ull);
-        for (int s = 0; s < kLzStages; ++s)
+        for (int s = 0; s < a.stages; ++s)
             if (prod.pending >> s & 1u) lz_mbar_wait(lz_saddr(&H.bar_full[s]), (prod.ipar >> s & 1u) ^ 1u);
     }
 }
 
-template <int G, int NV, bool SX, bool TMA = false>
-__global__ void __launch_bounds__(kLzThreads, 1) k_lz(Geo g, LzArgs a)
+template <int G, int NV, bool SX, int ST, bool TMA = false>
+__global__ void __launch_bounds__(lz_threads(ST), 1) k_lz(const __grid_constant__ Geo g, const __grid_constant__ LzArgs a)
 {
     extern __shared__ __align__(16) char smem_raw[];
     const int ngroups = (g.nr + G - 1) / G;
     const int nmine = blockIdx.x < ngroups ? (ngroups - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    lz_run<G, NV, SX, TMA>(g, a, smem_raw, blockIdx.x, gridDim.x, nmine);
+    lz_run<G, NV, SX, ST, TMA>(g, a, smem_raw, blockIdx.x, gridDim.x, nmine);
 }
 
 }  // namespace bzk
