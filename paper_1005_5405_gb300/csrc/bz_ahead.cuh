@@ -72,7 +72,7 @@ __global__ void k_ahead_plan(Geo g, AheadPlans A, int64_t step0)
 __global__ void __launch_bounds__(1024) k_ahead_scan(AheadPlans A, int64_t step0)
 {
     const int s = ahead_slot(A, step0, blockIdx.x);
-    const int64_t v = (int64_t)s * A.nvt, w = (int64_t)s * (A.nvt / 32);
+    const int64_t v = (int64_t)s * A.nvt, w = (int64_t)s * ((A.nvt + 31) / 32);
     lz_scan_block(A.nvt, A.mcap, A.flag + v, A.cidx + v, A.act + v, A.mask + w, A.wpre + w,
                   A.meta + s * kLzMetaSize, nullptr);
 }
@@ -120,12 +120,12 @@ __device__ __forceinline__ void ahead_take(const AheadPlans &A, int64_t step, in
     const int s = (int)(step % A.K);
     const int *sm = A.meta + s * kLzMetaSize;
     const int M = min(sm[0], A.nvt), C = sm[3];
-    const int64_t t0 = (int64_t)s * A.nt, v0 = (int64_t)s * A.nvt, w0 = (int64_t)s * (A.nvt / 32);
+    const int64_t t0 = (int64_t)s * A.nt, v0 = (int64_t)s * A.nvt, w0 = (int64_t)s * ((A.nvt + 31) / 32);
     for (int64_t i = i0; i < A.nt; i += stride) {
         idx[i] = A.idx[t0 + i];
         pa[i] = A.pa[t0 + i];
     }
-    for (int64_t i = i0; i < A.nvt / 32; i += stride) {
+    for (int64_t i = i0; i < (A.nvt + 31) / 32; i += stride) {
         mask[i] = A.mask[w0 + i];
         wpre[i] = A.wpre[w0 + i];
     }

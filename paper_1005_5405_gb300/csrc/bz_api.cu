@@ -423,7 +423,7 @@ double lz_monomial(int k, double x, double y, double z)
 // the kernel that reads it at run time); stretched grids (per-cell Courant
 // factors) have their own instances, specialised for 20 nodes per axis (the
 // paper's stretched cavities) and run-time lengths otherwise.
-int lz_nv_key(const bz_handle *H) { return H->stretched ? (H->g.nv == 20 ? -20 : -1) : H->g.nv; }
+int lz_nv_key(const bz_handle *H) { return H->stretched ? (H->g.nv == 20 || H->g.nv == 18 ? -H->g.nv : -1) : H->g.nv; }
 
 // Calls f with the k_lz instance of a handle: G cells per group, the axis
 // length as a constant where it has an instance, stretched cells, the
@@ -434,6 +434,11 @@ auto with_lz_kernel(const bz_handle *H, F f)
     if constexpr (G == 4 && ST == 256) {
         if (H->lz_tma && lz_nv_key(H) >= 0)
             return lz_nv_key(H) == 32 ? f(bzk::k_lz<4, 32, false, 256, true>) : f(bzk::k_lz<4, 0, false, 256, true>);
+    }
+    if (H->g.nv % 4 != 0) {
+        if constexpr (G == 4 && ST == 512)
+            if (lz_nv_key(H) == -18) return f(bzk::k_lz<4, 18, true, 512>);
+        return H->stretched ? f(bzk::k_lz<G, 0, true, ST, false, 2>) : f(bzk::k_lz<G, 0, false, ST, false, 2>);
     }
     if constexpr (G == 4 && ST == 512) {
         if (lz_nv_key(H) == 24) return f(bzk::k_lz<4, 24, false, 512>);
@@ -456,15 +461,17 @@ bz_status setup_lz_kernel(bz_handle *H, int G, int ST, size_t smem, int *occ)
         BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, bzk::lz_threads(ST), smem));
         return BZ_OK;
     };
-    if (ST == 512) return with_lz_kernel<4, 512>(H, set);
+    if (ST == 512) return G == 4 ? with_lz_kernel<4, 512>(H, set) : with_lz_kernel<2, 512>(H, set);
     return G == 4 ? with_lz_kernel<4, 256>(H, set) : with_lz_kernel<2, 256>(H, set);
 }
 
 void launch_lz_kernel(bz_handle *H, const bzk::LzArgs &a, cudaStream_t s)
 {
     auto go = [&](auto *k) { k<<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); };
-    if (H->lz_T == bzk::lz_threads(512)) with_lz_kernel<4, 512>(H, go);
-    else if (H->lz_G == 4) with_lz_kernel<4, 256>(H, go);
+    if (H->lz_T == bzk::lz_threads(512)) {
+        if (H->lz_G == 4) with_lz_kernel<4, 512>(H, go);
+        else with_lz_kernel<2, 512>(H, go);
+    } else if (H->lz_G == 4) with_lz_kernel<4, 256>(H, go);
     else with_lz_kernel<2, 256>(H, go);
 }
 
@@ -480,9 +487,12 @@ bz_status configure_lazy(bz_handle *H)
     const Geo &g = H->g;
     const char *force = getenv("BZ_KERNEL");
     if (force && (strcmp(force, "generic") == 0 || strcmp(force, "cell4") == 0)) return BZ_OK;
-    if (!H->fast || g.nv > bzk::kLzMaxN || g.nv % 4 != 0 || g.nvt % 32 != 0) return BZ_OK;
     const int N = g.nv, nvt = g.nvt, nt = g.nt;
-    if (bzk::lz_planes4(N, 256) == 0) return BZ_OK;
+    // Multiples of four nodes where the 4-node-vector kernel (the fallback)
+    // runs; N = 2 mod 4 from 14 on with the generic kernel as fallback.
+    const bool pairs = N % 4 == 2 && N >= 14 && H->dtype == BZ_F32 && !H->per_cell && H->idx16 && nt <= 32768;
+    if (!(H->fast || pairs) || N > bzk::kLzMaxN) return BZ_OK;
+    if (bzk::lz_planes(N, 512) == 0) return BZ_OK;
     const size_t mub = sizeof(float) * 8 * (size_t)g.nr;
     BZ_TRY(dalloc(&H->mu[0], mub));
     BZ_TRY(dalloc(&H->mu[1], mub));
@@ -494,8 +504,8 @@ bz_status configure_lazy(bz_handle *H)
     BZ_TRY(dalloc(&H->lz_flag, sizeof(int) * nvt));
     BZ_TRY(dalloc(&H->lz_cidx, sizeof(int) * nvt));
     BZ_TRY(dalloc(&H->lz_act, sizeof(int) * nvt));
-    BZ_TRY(dalloc(&H->lz_mask, sizeof(uint32_t) * (nvt / 32)));
-    BZ_TRY(dalloc(&H->lz_wpre, sizeof(int) * (nvt / 32)));
+    BZ_TRY(dalloc(&H->lz_mask, sizeof(uint32_t) * ((nvt + 31) / 32)));
+    BZ_TRY(dalloc(&H->lz_wpre, sizeof(int) * ((nvt + 31) / 32)));
     BZ_TRY(dalloc(&H->lz_meta, sizeof(int) * bzk::kLzMetaSize));
     BZ_CUDA(cudaMemset(H->lz_flag, 0, sizeof(int) * nvt));
     BZ_CUDA(cudaMemset(H->lz_meta, 0, sizeof(int) * bzk::kLzMetaSize));
@@ -533,18 +543,19 @@ bz_status configure_lazy(bz_handle *H)
     bool ok = false;
     const char *force_g = getenv("BZ_LAZY_G");
     const char *force_st = getenv("BZ_LAZY_ST");
-    for (const int ST : {512, 256}) {
-        for (const int G : {4, 2}) {
+    for (const int G : {4, 2}) {
+        for (const int ST : {512, 256}) {
             if (ok || (force_g && atoi(force_g) != G) || (force_st && atoi(force_st) != ST)) continue;
-            if (ST == 512 && (G != 4 || (!force_st && bzk::lz_stream_threads(N) != 512) || H->lz_tma)) continue;
+            if (ST == 512 && ((!force_st && bzk::lz_stream_threads(N) != 512) || H->lz_tma)) continue;
             // Term records address a compact array with 16-bit byte offsets.
             if ((size_t)mcap * 4 * G > 65535) continue;
             // As many streaming stages as fit (the copies in flight per SM).
-            const int S = bzk::lz_planes4(N, ST) * (N * N / 4);
+            const int VW = bzk::lz_vec(N), S = bzk::lz_planes(N, ST) * (N * N / VW);
+            if (S == 0 || (pairs && H->lz_tma)) continue;
             int stages = bzk::kLzMaxStages;
-            while (stages >= 3 && bzk::lz_offsets(nvt, mcap, G, stages, S).end > (size_t)H->smem_optin) --stages;
+            while (stages >= 3 && bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end > (size_t)H->smem_optin) --stages;
             if (stages < 3) continue;
-            const size_t smem = bzk::lz_offsets(nvt, mcap, G, stages, S).end;
+            const size_t smem = bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end;
             int occ = 0;
             BZ_TRY(setup_lz_kernel(H, G, ST, smem, &occ));
             if (occ < 1) continue;
@@ -638,8 +649,8 @@ bz_status configure_lazy(bz_handle *H)
         BZ_TRY(dalloc(&A.flag, sizeof(int) * k * nvt));
         BZ_TRY(dalloc(&A.cidx, sizeof(int) * k * nvt));
         BZ_TRY(dalloc(&A.act, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.mask, sizeof(uint32_t) * k * (nvt / 32)));
-        BZ_TRY(dalloc(&A.wpre, sizeof(int) * k * (nvt / 32)));
+        BZ_TRY(dalloc(&A.mask, sizeof(uint32_t) * k * ((nvt + 31) / 32)));
+        BZ_TRY(dalloc(&A.wpre, sizeof(int) * k * ((nvt + 31) / 32)));
         BZ_TRY(dalloc(&A.meta, sizeof(int) * k * bzk::kLzMetaSize));
         BZ_TRY(dalloc(&A.count, sizeof(int) * k * nvt));
         BZ_TRY(dalloc(&A.cursor, sizeof(int) * k * nvt));
@@ -835,28 +846,37 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
         bzk::k_lz_fb_plan<<<pg, pb, 0, s>>>(g.nt, g.nv, H->lz_meta, H->lz_idx, H->lz_pa,
                                             (ushort4 *)H->pidx, pa16, H->sc_count);
         BZ_LAUNCHED(H);
-        bzk::k_scatter_scan<<<1, 1024, 0, s>>>(g.nvt, H->threads4, H->sc_count, H->sc_cursor,
-                                               H->sc_meta, H->lz_meta);
-        BZ_LAUNCHED(H);
-        bzk::k_scatter_fill<<<pg, pb, 0, s>>>(g.nt, H->threads4, pi, H->sc_cursor, H->sc_meta,
-                                              H->sc_ent, H->lz_meta);
-        BZ_LAUNCHED(H);
+        if (H->fast) {
+            bzk::k_scatter_scan<<<1, 1024, 0, s>>>(g.nvt, H->threads4, H->sc_count, H->sc_cursor,
+                                                   H->sc_meta, H->lz_meta);
+            BZ_LAUNCHED(H);
+            bzk::k_scatter_fill<<<pg, pb, 0, s>>>(g.nt, H->threads4, pi, H->sc_cursor, H->sc_meta,
+                                                  H->sc_ent, H->lz_meta);
+            BZ_LAUNCHED(H);
+        }
         // The input is corrected in place and its pending corrections go;
         // the output's are cleared (k_cell4 writes corrected values).
         bzk::k_lz_materialize<<<std::min(g.nr, H->nsm * 8), 256, 0, s>>>(
             g, H->lz_meta, hin, H->mu[in], hin, H->mu[out], H->mu[in]);
         BZ_LAUNCHED(H);
         const int grid = nostream ? H->grid4c : H->grid4f;
+#define BZ_CG(F, gr)                                                                                  \
+    bzk::k_cell<float, F, uint16_t><<<gr, H->threads, H->smem_cell, s>>>(                             \
+        g, hin, (const float *)H->ghost, pi, pa16, (float *)H->gw_global, hout, H->mom, H->stats,     \
+        H->gw_in_smem, nullptr, H->lz_meta)
 #define BZ_C4G(F, M)                                                                              \
     bzk::k_cell4<F, M><<<grid, H->threads4, H->smem4, s>>>(g, H->map, hin, (const float *)H->ghost, \
                                                           pa16, H->sc_ent, H->sc_meta, hout, H->mom, \
                                                           H->stats, nullptr, H->lz_meta)
-        if (H->maxt4 == 512) {
+        if (!H->fast) {
+            if (nostream) BZ_CG(false, H->grid_cell); else BZ_CG(true, H->grid_cell_fused);
+        } else if (H->maxt4 == 512) {
             if (nostream) BZ_C4G(false, 512); else BZ_C4G(true, 512);
         } else {
             if (nostream) BZ_C4G(false, 1024); else BZ_C4G(true, 1024);
         }
 #undef BZ_C4G
+#undef BZ_CG
         BZ_LAUNCHED(H);
     }
     if (!advance_step) return BZ_OK;           // a repeatable trial of the step

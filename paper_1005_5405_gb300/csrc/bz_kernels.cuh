@@ -941,8 +941,9 @@ k_cell(Geo g, const R *__restrict__ hin, const R *__restrict__ ghost,
        const typename Idx4<I>::type *__restrict__ pidx, const PlanA<R, I> *__restrict__ pa,
        R *__restrict__ gw_global,
        R *__restrict__ hout, double *__restrict__ mom, unsigned long long *__restrict__ stats,
-       int gw_in_smem, const int64_t *__restrict__ stepp = nullptr)
+       int gw_in_smem, const int64_t *__restrict__ stepp = nullptr, const int *__restrict__ gate = nullptr)
 {
+    if (gate && !gate[1]) return;            // the active-node kernel's fallback: only when it gave up
     extern __shared__ __align__(16) char smem_raw[];
     CellSmem<R> S = carve<R>(smem_raw, g, gw_in_smem != 0);
     using V4 = typename Idx4<I>::type;

@@ -66,24 +66,30 @@ constexpr unsigned long long kLzWaitNs = 1000000000ull;   // an mbarrier wait gi
 // [3] C (terms per thread).
 constexpr int kLzMetaSize = 4;
 
-// Planes per streaming stage: the largest divisor K of N/2 with K N^2/4 <=
-// ST (one node quad per streaming thread; stages never straddle jx =
+// Nodes per streaming thread and stage: four consecutive jz (16-byte loads
+// and stores), or two where rows of N nodes are not multiples of 16 bytes
+// (N = 2 mod 4; before, such grids ran the generic per-cell kernel: ten steps of
+// 192^2 x 18^3, stretched, 8192 samples, 45.4 -> 17.2 ms).
+__host__ __device__ constexpr int lz_vec(int N) { return N % 4 == 0 ? 4 : 2; }
+
+// Planes per streaming stage: the largest divisor K of N/2 with K N^2/VW <=
+// ST (one node vector per streaming thread; stages never straddle jx =
 // N/2, so the upwind x source is the same cell for the whole stage).  0:
 // unsupported.
-__host__ __device__ constexpr int lz_planes4(int N, int ST)
+__host__ __device__ constexpr int lz_planes(int N, int ST)
 {
     int K = 0;
     for (int k = 1; k <= N / 2; ++k)
-        if ((N / 2) % k == 0 && k * (N * N / 4) <= ST) K = k;
+        if ((N / 2) % k == 0 && k * (N * N / lz_vec(N)) <= ST) K = k;
     return K;
 }
 
 // Streaming threads for N nodes per axis: 512 where that raises the busy
-// share by more than 1.4 (above), else 256.
+// share by more than 1.4 (above), or where a plane needs them, else 256.
 constexpr int lz_stream_threads(int N)
 {
-    const int q = N * N / 4, s2 = lz_planes4(N, 256) * q, s5 = lz_planes4(N, 512) * q;
-    return 10 * s5 * 256 > 14 * s2 * 512 ? 512 : 256;
+    const int s2 = lz_planes(N, 256), s5 = lz_planes(N, 512);
+    return s2 == 0 || 10 * s5 * 256 > 14 * s2 * 512 ? 512 : 256;
 }
 
 // ---------------------------------------------------------------------
@@ -116,7 +122,7 @@ __device__ __forceinline__ void lz_scan_block(int nvt, int mcap, int *__restrict
 {
     __shared__ int wsum[32];
     __shared__ int btot;
-    const int t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = nvt / 32;
+    const int t = threadIdx.x, lane = t & 31, wp = t >> 5, nw = (nvt + 31) / 32;
     int carry = 0;
     for (int b0 = 0; b0 < nw; b0 += 1024) {
         const int base = b0 + wp * 32;                // this warp's 32 words
@@ -124,7 +130,7 @@ __device__ __forceinline__ void lz_scan_block(int nvt, int mcap, int *__restrict
 #pragma unroll 8
         for (int k = 0; k < 32; ++k) {
             const int w = base + k;
-            const bool set = w < nw && flag[w * 32 + lane] != 0;
+            const bool set = w * 32 + lane < nvt && flag[w * 32 + lane] != 0;
             const uint32_t bal = __ballot_sync(0xFFFFFFFFu, set);
             if (lane == k) bits = bal;
         }
@@ -530,9 +536,11 @@ __global__ void __launch_bounds__(32) k_lz_order(int T, int cmax, int chunk, con
 }
 
 // ---------------------------------------------------------------------
-// Fallback when a step has more active nodes than mcap: the k_cell4 plan is
+// Fallback when a step has more active nodes than mcap: the k_cell4 plan (or,
+// for N = 2 mod 4, that of the generic kernel, in logical node order) is
 // derived from the logical one, the input is corrected in place and mu_out
-// is cleared (k_cell4 writes corrected states).  All return at once otherwise.
+// is cleared (those kernels write corrected states).  All return at once
+// otherwise.
 // ---------------------------------------------------------------------
 __device__ __forceinline__ void lz_fb_plan_one(int l, int N, const int4 *__restrict__ idx,
                                                const PlanA<float, int> *__restrict__ pa,
@@ -545,7 +553,7 @@ __device__ __forceinline__ void lz_fb_plan_one(int l, int N, const int4 *__restr
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int j = o[k];
-        if (j < 0) continue;
+        if (j < 0 || N % 4 != 0) continue;
         const int jx = j / (N * N), jz = j % N, row = j - jz;
         int r = jz / 4 + jx % nq;
         if (r >= nq) r -= nq;
@@ -554,6 +562,7 @@ __device__ __forceinline__ void lz_fb_plan_one(int l, int N, const int4 *__restr
     const ushort4 u = Idx4<uint16_t>::make(o);
     pidx16[l] = u;
     pa16[l] = make_plan_a<float, uint16_t>(o[0], o[1], (double)pa[l].W);
+    if (!count) return;
     if (u.x != 0xFFFF) atomicAdd(count + u.x, 1);
     if (u.y != 0xFFFF) atomicAdd(count + u.y, 1);
     if (u.z != 0xFFFF) atomicAdd(count + u.z, 1);
@@ -582,6 +591,7 @@ static __global__ void k_lz_materialize(Geo g, const int *__restrict__ skip_unle
     __shared__ float sv[kMaxN];
     __shared__ float smu[8];
     const int N = g.nv, nq = N / 4, Q = N * N / 4;
+    const bool rows4 = N % 4 == 0;                   // a float4 lies in one row
     for (int i = threadIdx.x; i < N; i += blockDim.x) sv[i] = (float)g.axv[i];
     const float eps = g.epsf;
     const int64_t plane = g.nvt / 4;
@@ -593,13 +603,21 @@ static __global__ void k_lz_materialize(Geo g, const int *__restrict__ skip_unle
         const float4 *src = reinterpret_cast<const float4 *>(hin) + (int64_t)c * plane;
         float4 *dst = reinterpret_cast<float4 *>(hout) + (int64_t)c * plane;
         for (int o = threadIdx.x; o < (int)plane; o += blockDim.x) {
-            const int jx = o / Q, q = o % Q, jy = q / nq, jz = 4 * (q % nq);
-            const float vx = sv[jx], vy = sv[jy];
             float4 h = src[o];
             float *hp = &h.x;
+            if (rows4) {
+                const int jx = o / Q, q = o % Q, jy = q / nq, jz = 4 * (q % nq);
+                const float vx = sv[jx], vy = sv[jy];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                hp[i] = state_corr(hp[i], state_kappa(smu, vx, vy, sv[jz + i]), eps);
+                for (int i = 0; i < 4; ++i) hp[i] = state_corr(hp[i], state_kappa(smu, vx, vy, sv[jz + i]), eps);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; i += 2) {     // (two nodes of a row)
+                    const int j = 4 * o + i, jxy = j / N, jx = jxy / N, jz = j - jxy * N;
+                    const float vx = sv[jx], vy = sv[jxy - jx * N];
+                    hp[i] = state_corr(hp[i], state_kappa(smu, vx, vy, sv[jz]), eps);
+                    hp[i + 1] = state_corr(hp[i + 1], state_kappa(smu, vx, vy, sv[jz + 1]), eps);
+                }
             }
             dst[o] = h;
         }
@@ -793,15 +811,15 @@ constexpr uint32_t kLzAOff = (sizeof(LzHead) + 15) & ~(size_t)15;
 struct LzOff {
     uint32_t abytes, a1, bc, ring, mask, act, end;
 };
-__host__ __device__ inline LzOff lz_offsets(int nvt, int mcap, int G, int stages, int S)
+__host__ __device__ inline LzOff lz_offsets(int nvt, int mcap, int G, int stages, int S, int VW)
 {
     LzOff o;
     o.abytes = (uint32_t)(((sizeof(float) * (size_t)G * (mcap + 1)) + 127) & ~(size_t)127);
     size_t off = kLzAOff + o.abytes;
     o.a1 = (uint32_t)off; off += o.abytes;
     o.bc = (uint32_t)off; off += o.abytes;
-    o.ring = (uint32_t)off; off += (size_t)stages * 3 * S * sizeof(float4);
-    o.mask = (uint32_t)off; off += sizeof(uint2) * (nvt / 32);
+    o.ring = (uint32_t)off; off += (size_t)stages * 3 * S * VW * sizeof(float);
+    o.mask = (uint32_t)off; off += sizeof(uint2) * ((nvt + 31) / 32);
     o.act = (uint32_t)off; off += sizeof(uint16_t) * (size_t)mcap;
     o.end = (uint32_t)((off + 15) & ~(size_t)15);
     return o;
@@ -976,20 +994,20 @@ __device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, 
     if (lane < 11) a.mom[(int64_t)c * 11 + lane] = (double)o;
 }
 
-// The (v_y, v_z) part of a cell's pending correction at a thread's four
-// nodes (jy, 4 qz .. 4 qz + 3): mu_y v_y + mu_z v_z + mu_4 (v_y^2 + v_z^2), as
-// two node pairs.
-__device__ __forceinline__ void lz_bd(const float *mu, const float *v, int jy, int qz, float2 (&bd)[2])
+// The (v_y, v_z) part of a cell's pending correction at a thread's nodes (jy;
+// jz .. jz + VW - 1): mu_y v_y + mu_z v_z + mu_4 (v_y^2 + v_z^2), as node pairs.
+template <int VW>
+__device__ __forceinline__ void lz_bd(const float *mu, const float *v, int jy, int jz, float2 (&bd)[VW / 2])
 {
     const float vy = v[jy];
-    float b[4];
+    float b[VW];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float vz = v[4 * qz + i];
+    for (int i = 0; i < VW; ++i) {
+        const float vz = v[jz + i];
         b[i] = mu[2] * vy + mu[3] * vz + mu[4] * (vy * vy + vz * vz);
     }
-    bd[0] = make_float2(b[0], b[1]);
-    bd[1] = make_float2(b[2], b[3]);
+#pragma unroll
+    for (int p = 0; p < VW / 2; ++p) bd[p] = make_float2(b[2 * p], b[2 * p + 1]);
 }
 
 // lz_mono_from_powers for two cells at once (s and M hold one value per
@@ -1056,6 +1074,33 @@ __device__ __forceinline__ void lz_sts4(uint32_t dst, float v)
 {
     asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(v) : "memory");
 }
+__device__ __forceinline__ void lz_cp8s(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void lz_sts2(uint32_t dst, float v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %1};" ::"r"(dst), "f"(v) : "memory");
+}
+__device__ __forceinline__ float2 lz_lds2(uint32_t src)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(src) : "memory");
+    return v;
+}
+// A thread's node vector: VW = 4 or 2 values.
+template <int VW>
+__device__ __forceinline__ void lz_cps(uint32_t dst, const void *src)
+{
+    if (VW == 4) lz_cp16s(dst, src);
+    else lz_cp8s(dst, src);
+}
+template <int VW>
+__device__ __forceinline__ void lz_stsv(uint32_t dst, float v)
+{
+    if (VW == 4) lz_sts4(dst, v);
+    else lz_sts2(dst, v);
+}
 __device__ __forceinline__ float4 lz_lds4(uint32_t src)
 {
     float4 v;
@@ -1071,9 +1116,9 @@ struct LzQuad {
     int S, J, Jh, P4, pl, N, jy;
     bool yup, streams;
     int64_t pbytes;             // bytes per cell (N^3 floats)
-    int sbytes;                 // bytes per stage of a cell (S float4)
+    int sbytes;                 // bytes per stage of a cell (S node vectors)
     uint32_t ring0, ring_end;   // shared addresses: this thread's slots of ring slot 0; ring end
-    uint32_t src;               // bytes between the three sources of a stage (S float4)
+    uint32_t src;               // bytes between the three sources of a stage
     int stages;
 };
 
@@ -1111,16 +1156,17 @@ __device__ __forceinline__ void lz_pf_cell(LzPf &p, const LzQuad &q, const Geo &
 // Stages this thread's own, x-source and y-source quads of the next stage
 // (a wall's ghost value where the source lies outside the cavity) and
 // commits one group of copies (an empty one past the group's last stage).
+template <int VW>
 __device__ __forceinline__ void lz_prefetch(LzPf &p, const LzQuad &q, const Geo &g, const LzArgs &a,
                                             const int4 *cells, const char *hin_t, int ncell)
 {
     if (q.streams && p.pk < ncell) {
         if (p.pst == 0) lz_pf_cell(p, q, g, a, cells, hin_t);
-        lz_cp16s(p.slot, p.own);
-        if (p.xin) lz_cp16s(p.slot + q.src, p.own + p.xoff);
-        else lz_sts4(p.slot + q.src, p.gx);
-        if (p.yin) lz_cp16s(p.slot + 2 * q.src, p.own + p.yoff);
-        else lz_sts4(p.slot + 2 * q.src, __ldg(p.gy + p.pst * q.P4));
+        lz_cps<VW>(p.slot, p.own);
+        if (p.xin) lz_cps<VW>(p.slot + q.src, p.own + p.xoff);
+        else lz_stsv<VW>(p.slot + q.src, p.gx);
+        if (p.yin) lz_cps<VW>(p.slot + 2 * q.src, p.own + p.yoff);
+        else lz_stsv<VW>(p.slot + 2 * q.src, __ldg(p.gy + p.pst * q.P4));
         p.own += q.sbytes;
     }
     lz_cp_commit();
@@ -1213,34 +1259,42 @@ __device__ __forceinline__ void lz_prefetch_tma(LzPf &p, const LzQuad &q, const 
 
 // Per-cell state of a thread's streaming: the (v_y, v_z) parts of the
 // sources' pending corrections and the power sums over jx of N = w h~ /
-// (A_y A_z) for the quad's two node pairs.
-struct LzAcc {
-    float2 bdo[2], bdx[2], bdy[2];
-    float2 s0[2], s1[2], s2[2], s3[2], s4[2];
+// (A_y A_z) for the vector's node pairs.
+template <int VW> struct LzAcc {
+    float2 bdo[VW / 2], bdx[VW / 2], bdy[VW / 2];
+    float2 s0[VW / 2], s1[VW / 2], s2[VW / 2], s3[VW / 2], s4[VW / 2];
 };
 
 // One streaming stage of one cell (Eq. streaming2D with the deferred
 // correction applied to its sources): h~ to dst, the power sums, and the
 // active nodes of the quad to the compact array (component k of G).  SX:
 // stretched cells, the x Courant numbers times the cell's factor fx2.
-template <int G, bool SX>
+template <int G, bool SX, int VW>
 __device__ __forceinline__ void lz_stream_stage(uint32_t sl, uint32_t src, int jx, int j0, int k, const LzHead &H,
-                                                const float4 *tcx, const float2 *tcy, LzAcc &c,
-                                                float4 *dst, const uint2 *smask, float *Af,
+                                                const float4 *tcx, const float2 *tcy, LzAcc<VW> &c,
+                                                char *dst, const uint2 *smask, float *Af,
                                                 float2 eps2, float2 one2, float2 nay2, float2 fx2)
 {
-    const float4 h0 = lz_lds4(sl), hx = lz_lds4(sl + src), hy = lz_lds4(sl + 2 * src);
+    float2 h0p[VW / 2], hxp[VW / 2], hyp[VW / 2];
+    if constexpr (VW == 4) {
+        const float4 h0 = lz_lds4(sl), hx = lz_lds4(sl + src), hy = lz_lds4(sl + 2 * src);
+        h0p[0] = lz_lo(h0); h0p[1] = lz_hi(h0);
+        hxp[0] = lz_lo(hx); hxp[1] = lz_hi(hx);
+        hyp[0] = lz_lo(hy); hyp[1] = lz_hi(hy);
+    } else {
+        h0p[0] = lz_lds2(sl);
+        hxp[0] = lz_lds2(sl + src);
+        hyp[0] = lz_lds2(sl + 2 * src);
+    }
     const float4 cx4 = tcx[jx];
     const float2 cy2 = tcy[jx];
     const float4 ta = H.ta[jx];
     const float2 nax2 = SX ? lz_mul2(lz_lo(ta), fx2) : lz_lo(ta), A2 = lz_hi(ta);
     const float4 v12 = H.tv12[jx], v34 = H.tv34[jx];
-    const float2 h0p[2] = {lz_lo(h0), lz_hi(h0)}, hxp[2] = {lz_lo(hx), lz_hi(hx)},
-                 hyp[2] = {lz_lo(hy), lz_hi(hy)};
-    float2 ht[2];
+    float2 ht[VW / 2];
     const float2 mone2 = lz_dup(-1.f);
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
+    for (int p = 0; p < VW / 2; ++p) {
         // u = h_c + (1 + eps h_c) kappa of each source, as h_c (1 + eps kappa) + kappa.
         const float2 ko = lz_add2(lz_lo(cx4), c.bdo[p]);
         const float2 u0 = lz_fma2(h0p[p], lz_fma2(eps2, ko, one2), ko);
@@ -1259,17 +1313,17 @@ __device__ __forceinline__ void lz_stream_stage(uint32_t sl, uint32_t src, int j
         c.s3[p] = lz_fma2(n, lz_lo(v34), c.s3[p]);
         c.s4[p] = lz_fma2(n, lz_hi(v34), c.s4[p]);
     }
-    *dst = make_float4(ht[0].x, ht[0].y, ht[1].x, ht[1].y);
+    if constexpr (VW == 4) *reinterpret_cast<float4 *>(dst) = make_float4(ht[0].x, ht[0].y, ht[1].x, ht[1].y);
+    else *reinterpret_cast<float2 *>(dst) = ht[0];
     // Active nodes of the quad (nodes j0 .. j0 + 3) go to the compact array.
     const uint2 mw = smask[j0 >> 5];
     const int sh = j0 & 31;
-    const uint32_t bits = (mw.x >> sh) & 15u;
+    const uint32_t bits = (mw.x >> sh) & ((1u << VW) - 1u);
     if (bits) {
         int mi = (int)mw.y + __popc(mw.x & ((1u << sh) - 1u));
-        const float hv[4] = {ht[0].x, ht[0].y, ht[1].x, ht[1].y};
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (bits >> i & 1u) Af[(mi++) * G + k] = hv[i];
+        for (int i = 0; i < VW; ++i)
+            if (bits >> i & 1u) Af[(mi++) * G + k] = i & 1 ? ht[i / 2].y : ht[i / 2].x;
     }
 }
 
@@ -1378,7 +1432,7 @@ constexpr int kLzTailChunk = 256;  // active nodes per claimed chunk of the incr
 // lz_run runs the pipeline of one CTA over the groups grp0, grp0 + gstride,
 // ... (nmine of them) of one problem; the kernel k_lz gives CTA b the groups
 // b, b + gridDim.x, ...
-template <int G, int NV, bool SX, int ST, bool TMA = false>
+template <int G, int NV, bool SX, int ST, bool TMA = false, int VW = NV % 4 == 0 ? 4 : 2>
 __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem_raw, int grp0, int gstride,
                                        int nmine)
 {
@@ -1392,14 +1446,12 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
     }
     const int N = NV ? NV : g.nv;
     const int N2 = N * N, nvt = N2 * N, t = threadIdx.x;
-    const int Qd = N2 / 4, nq = N / 4, P4 = lz_planes4(N, ST), J = N / P4, Jh = J / 2;
-    const int S = P4 * Qd;                        // float4 per stage (the threads that stream)
+    const int Qd = N2 / VW, nq = N / VW, P4 = lz_planes(N, ST), J = N / P4, Jh = J / 2;
+    const int S = P4 * Qd;                        // node vectors per stage (the threads that stream)
     const int half = N / 2;
-    const int64_t plane4 = nvt / 4;               // float4 per cell
     LzHead &H = *reinterpret_cast<LzHead *>(smem_raw);
     const int M = a.meta[0];
-    const LzOff so = lz_offsets(nvt, a.mcap, G, a.stages, S);
-    float4 *ring = reinterpret_cast<float4 *>(smem_raw + so.ring);
+    const LzOff so = lz_offsets(nvt, a.mcap, G, a.stages, S, VW);
     V *Bv = reinterpret_cast<V *>(smem_raw + so.bc);
     float *Bf = reinterpret_cast<float *>(smem_raw + so.bc);
     uint2 *smask = reinterpret_cast<uint2 *>(smem_raw + so.mask);   // mask word, compact index of its first node
@@ -1424,7 +1476,7 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
         H.tv12[i] = make_float4(fv, fv, v2, v2);
         H.tv34[i] = make_float4(v3, v3, v4, v4);
     }
-    for (int w = t; w < nvt / 32; w += kThreads) {
+    for (int w = t; w < (nvt + 31) / 32; w += kThreads) {
         smask[w] = make_uint2(a.mask[w], (uint32_t)a.wpre[w]);
     }
     for (int m = t; m < M; m += kThreads) {     // active nodes as jx << 10 | jy << 5 | jz
@@ -1447,11 +1499,9 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
     // A streaming thread's quad.
     const bool streams = t < S;
     const int pl = streams ? t / Qd : 0, q = streams ? t - pl * Qd : 0;
-    const int jy = q / nq, qz = q - jy * nq;
+    const int jy = q / nq, jz = VW * (q - jy * nq);
     const bool yup = jy >= half;                  // v_y > 0: the y source is below
     const float2 nay2 = lz_dup(-H.cuy[jy]);
-    const float4 *hin4 = reinterpret_cast<const float4 *>(a.hin);
-    float4 *hout4 = reinterpret_cast<float4 *>(a.hout);
     int fallback = 0;
     LzTmaProd prod{0u, 0u, 0u};                   // thread 0: the bulk-copy ring's producer state
     uint32_t fpar = 0u;                           // parity of each slot's next full phase
@@ -1516,17 +1566,17 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     H.mus[k][s5][m] = ok ? a.mu_in[(int64_t)cs * 8 + m] : 0.f;
                 }
                 // a.stages - 1 stages in flight ahead of the one being used.
-                const uint32_t ring0 = lz_saddr(ring) + t * 16;
-                const LzQuad qd{S, J, Jh, P4, pl, N, jy, yup, streams, (int64_t)nvt * 4, S * 16, ring0,
-                                ring0 + a.stages * 3 * S * 16, (uint32_t)(S * 16), a.stages};
-                const char *hin_t = reinterpret_cast<const char *>(hin4 + t);
+                const uint32_t ring0 = lz_saddr(smem_raw + so.ring) + t * (VW * 4);
+                const LzQuad qd{S, J, Jh, P4, pl, N, jy, yup, streams, (int64_t)nvt * 4, S * VW * 4, ring0,
+                                ring0 + a.stages * 3 * S * VW * 4, (uint32_t)(S * VW * 4), a.stages};
+                const char *hin_t = reinterpret_cast<const char *>(a.hin) + t * (VW * 4);
                 LzPf pf{};
                 pf.slot = ring0;
                 const int4 *cells = H.cell[buf];
 #pragma unroll 1
                 for (int kk = 0; kk < a.stages - 1; ++kk) {
                     if (TMA) lz_prefetch_tma(pf, qd, g, a, cells, hin_t, ncell, H, prod);
-                    else lz_prefetch(pf, qd, g, a, cells, hin_t, ncell);
+                    else lz_prefetch<VW>(pf, qd, g, a, cells, hin_t, ncell);
                 }
                 lz_stream_bar<ST>();
                 // Correction tables of the group's cells: ca(jx) = mu_0 + mu_x
@@ -1557,26 +1607,26 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     // by the threads (generic proxy) before later bulk copies.
                     const int4 cek = cells[k];
                     const bool wallk = TMA && (cek.y == 0 || cek.y == g.nx - 1 || cek.z == 0 || cek.z == g.ny - 1);
-                    LzAcc ac;
+                    LzAcc<VW> ac;
 #pragma unroll
-                    for (int p = 0; p < 2; ++p)
+                    for (int p = 0; p < VW / 2; ++p)
                         ac.s0[p] = ac.s1[p] = ac.s2[p] = ac.s3[p] = ac.s4[p] = lz_zero2();
-                    lz_bd(H.mus[k][0], H.v, jy, qz, ac.bdo);
-                    lz_bd(H.mus[k][1], H.v, jy, qz, ac.bdx);
-                    lz_bd(H.mus[k][yup ? 3 : 4], H.v, jy, qz, ac.bdy);
+                    lz_bd<VW>(H.mus[k][0], H.v, jy, jz, ac.bdo);
+                    lz_bd<VW>(H.mus[k][1], H.v, jy, jz, ac.bdx);
+                    lz_bd<VW>(H.mus[k][yup ? 3 : 4], H.v, jy, jz, ac.bdy);
                     const float4 *tcx = H.tcx[k];
                     const float2 *tcy = H.tcy[k][yup ? 0 : 1];
-                    float4 *dst = hout4 + (int64_t)cells[k].x * plane4 + t;
+                    char *dst = reinterpret_cast<char *>(a.hout) + (int64_t)cells[k].x * nvt * 4 + t * (VW * 4);
                     // Courant factors of this cell on stretched grids.
                     float2 fx2 = one2, nay2k = nay2;
                     if (SX) {
                         fx2 = lz_dup((float)g.sx[cells[k].y]);
                         nay2k = lz_dup(-H.cuy[jy] * (float)g.sy[cells[k].z]);
                     }
-                    int jx = pl, j0 = 4 * t;
+                    int jx = pl, j0 = VW * t;
 #pragma unroll 1
                     for (int st = 0; st < J; ++st) {
-                        if (st == Jh) lz_bd(H.mus[k][2], H.v, jy, qz, ac.bdx);   // the left cell now
+                        if (st == Jh) lz_bd<VW>(H.mus[k][2], H.v, jy, jz, ac.bdx);   // the left cell now
                         // The slots read last stage take the stage a.stages - 1
                         // ahead; then this stage's copies have landed.
                         if (TMA) {
@@ -1584,11 +1634,11 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                             lz_ring_wait(lz_saddr(&H.bar_full[cidx]), fpar >> cidx & 1u, H.tma_err);
                             fpar ^= 1u << cidx;
                         } else {
-                            lz_prefetch(pf, qd, g, a, cells, hin_t, ncell);
+                            lz_prefetch<VW>(pf, qd, g, a, cells, hin_t, ncell);
                             lz_cp_wait_but(a.stages - 1);
                         }
                         if (streams)
-                            lz_stream_stage<G, SX>(cslot, qd.src, jx, j0, k, H, tcx, tcy, ac, dst, smask, Af,
+                            lz_stream_stage<G, SX, VW>(cslot, qd.src, jx, j0, k, H, tcx, tcy, ac, dst, smask, Af,
                                                    eps2, one2, nay2k, fx2);
                         if (TMA) {
                             // The warp has read the slot: release it to the producer.
@@ -1606,8 +1656,8 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                             cslot = ring0;
                         }
                         jx += P4;
-                        j0 += 4 * S;
-                        dst += S;
+                        j0 += VW * S;
+                        dst += S * VW * 4;
                     }
                     // The 26 monomial sums of the thread's nodes, summed over the warp.
                     float Msum[32];
@@ -1615,18 +1665,17 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                     for (int r = 0; r < 32; ++r) Msum[r] = 0.f;
                     if (streams) {
                         const float Ay = H.A[jy];
-                        const float sv[4][5] = {
-                            {ac.s0[0].x, ac.s1[0].x, ac.s2[0].x, ac.s3[0].x, ac.s4[0].x},
-                            {ac.s0[0].y, ac.s1[0].y, ac.s2[0].y, ac.s3[0].y, ac.s4[0].y},
-                            {ac.s0[1].x, ac.s1[1].x, ac.s2[1].x, ac.s3[1].x, ac.s4[1].x},
-                            {ac.s0[1].y, ac.s1[1].y, ac.s2[1].y, ac.s3[1].y, ac.s4[1].y}};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float Ayz = Ay * H.A[4 * qz + i];
+                        for (int i = 0; i < VW; ++i) {
+                            const int p = i / 2;
+                            const float Ayz = Ay * H.A[jz + i];
+                            const float sv[5] = {i & 1 ? ac.s0[p].y : ac.s0[p].x, i & 1 ? ac.s1[p].y : ac.s1[p].x,
+                                                 i & 1 ? ac.s2[p].y : ac.s2[p].x, i & 1 ? ac.s3[p].y : ac.s3[p].x,
+                                                 i & 1 ? ac.s4[p].y : ac.s4[p].x};
                             float si[5];
 #pragma unroll
-                            for (int pp = 0; pp < 5; ++pp) si[pp] = sv[i][pp] * Ayz;
-                            lz_mono_from_powers(si, H.v[jy], H.v[4 * qz + i], Msum);
+                            for (int pp = 0; pp < 5; ++pp) si[pp] = sv[pp] * Ayz;
+                            lz_mono_from_powers(si, H.v[jy], H.v[jz + i], Msum);
                         }
                     }
                     H.fpart[k][warp][lane] = lz_warp_reduce_scatter(Msum);
@@ -1839,13 +1888,13 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
     }
 }
 
-template <int G, int NV, bool SX, int ST, bool TMA = false>
+template <int G, int NV, bool SX, int ST, bool TMA = false, int VW = NV % 4 == 0 ? 4 : 2>
 __global__ void __launch_bounds__(lz_threads(ST), 1) k_lz(const __grid_constant__ Geo g, const __grid_constant__ LzArgs a)
 {
     extern __shared__ __align__(16) char smem_raw[];
     const int ngroups = (g.nr + G - 1) / G;
     const int nmine = blockIdx.x < ngroups ? (ngroups - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    lz_run<G, NV, SX, ST, TMA>(g, a, smem_raw, blockIdx.x, gridDim.x, nmine);
+    lz_run<G, NV, SX, ST, TMA, VW>(g, a, smem_raw, blockIdx.x, gridDim.x, nmine);
 }
 
 }  // namespace bzk
