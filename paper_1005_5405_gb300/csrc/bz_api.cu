@@ -11,6 +11,7 @@
 #include "bz_batch.cuh"
 #include "bz_lazy.cuh"
 #include "bz_ahead.cuh"
+#include "bz_relax.cuh"
 
 #include <cuda_runtime.h>
 
@@ -148,6 +149,18 @@ struct bz_handle {
     int lz_chunk = 0;                      // positions per chunk of the ordering
     cudaStream_t lz_side = nullptr;        // the sample plan runs here, beside the walls
     cudaEvent_t lz_fork = nullptr, lz_join = nullptr, lz_mid = nullptr;
+    // The cells with separate increments (bz_relax.cuh): FP64 states, odd axes
+    // and per-cell sets; its plans cover steps [rx_lo, rx_hi).
+    bool relax = false;
+    bool captured = false;              // the caller is capturing the stream: no plans built ahead
+    int rx_T = 0, rx_nseg = 1, rx_grid = 0, rx_K = 0, rx_minb = 1;
+    size_t rx_smem = 0;
+    void *rx_pa = nullptr;
+    ushort4 *rx_idx = nullptr;
+    int *rx_count = nullptr, *rx_cursor = nullptr, *rx_meta = nullptr;
+    uint32_t *rx_ent = nullptr;
+    unsigned long long *rx_cnt = nullptr;
+    int64_t rx_entn = 0, rx_lo = 0, rx_hi = 0;
     size_t lz_smem = 0;
     float lz_e0[bzk::kLzX] = {};
 };
@@ -688,6 +701,136 @@ bz_status configure_lazy(bz_handle *H)
     return BZ_OK;
 }
 
+// ---------------------------------------------------------------------
+// Cells with separate increments (bz_relax.cuh)
+// ---------------------------------------------------------------------
+template <typename R>
+bzk::RxPlans<R> rx_plans(const bz_handle *H)
+{
+    bzk::RxPlans<R> A{};
+    A.K = H->rx_K;
+    A.nt = H->g.nt;
+    A.nvt = H->g.nvt;
+    A.T = H->rx_T;
+    A.pa = (bzk::PlanA<R, uint16_t> *)H->rx_pa;
+    A.idx = H->rx_idx;
+    A.count = H->rx_count;
+    A.cursor = H->rx_cursor;
+    A.meta = H->rx_meta;
+    A.ent = H->rx_ent;
+    A.entn = H->rx_entn;
+    A.cnt = H->rx_cnt;
+    return A;
+}
+
+// Calls f with the k_relax instance of a handle.  FP64 has 512 threads at
+// most (32 sums of 8 bytes at the reduction), per-cell sets two CTAs of up to
+// 576 threads where two fit.
+template <typename R, bool FUSED, typename F>
+auto with_relax_kernel(const bz_handle *H, F f)
+{
+    if constexpr (sizeof(R) == 8) {
+        return H->per_cell ? f(bzk::k_relax<double, FUSED, true, 512, 1>) : f(bzk::k_relax<double, FUSED, false, 512, 1>);
+    } else {
+        if (!H->per_cell) return f(bzk::k_relax<float, FUSED, false, 1024, 1>);
+        return H->rx_minb == 2 ? f(bzk::k_relax<float, FUSED, true, 576, 2>) : f(bzk::k_relax<float, FUSED, true, 1024, 1>);
+    }
+}
+
+template <typename R>
+bz_status configure_relax(bz_handle *H)
+{
+    const Geo &g = H->g;
+    const int N = g.nv, N2 = N * N;
+    const int maxt = sizeof(R) == 8 ? 512 : 1024;
+    if (N2 > maxt) return BZ_OK;
+    // Segments of jx per column: to fill up to 512 threads where samples are
+    // drawn in the cell or FP32 does the sums; for FP64 (each segment repeats
+    // the 26 sums of its column) only where there are few cells per SM.
+    int nseg = 1;
+    if (H->per_cell || sizeof(R) == 4) nseg = std::max(1, 512 / N2);
+    else if (g.nr <= 4 * H->nsm) nseg = std::max(1, 448 / N2);
+    nseg = std::min(nseg, std::min(N, sizeof(R) == 8 ? 3 : 8));
+    H->rx_nseg = nseg;
+    H->rx_T = (N2 * nseg + 31) / 32 * 32;
+    H->rx_smem = bzk::rx_smem<R>(nullptr, nullptr, N, g.nvt, H->rx_T, H->per_cell ? 0 : g.nt);
+    if (H->rx_smem > (size_t)H->smem_optin) return BZ_OK;
+    H->rx_minb = sizeof(R) == 4 && H->per_cell && H->rx_T <= 576 ? 2 : 1;
+    int occ = 0;
+    auto set = [&](auto *k) -> bz_status {
+        int o = 0;
+        BZ_CUDA(bz_allow_max_smem(k, H->smem_optin));
+        BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, H->rx_T, H->rx_smem));
+        occ = occ ? std::min(occ, o) : o;
+        return BZ_OK;
+    };
+    BZ_TRY((with_relax_kernel<R, true>(H, set)));
+    BZ_TRY((with_relax_kernel<R, false>(H, set)));
+    if (occ < 1) return BZ_OK;
+    H->rx_grid = std::min(g.nr, H->nsm * occ);
+    if (!H->per_cell) {
+        // Plans of up to 32 steps (an even count, for the two-step graphs),
+        // within about 32 MiB.
+        const int64_t per = (int64_t)g.nt * (sizeof(bzk::PlanA<R, uint16_t>) + 8 + 16) + (int64_t)g.nvt * 8;
+        const int K = H->rx_K = (int)std::max<int64_t>(2, std::min<int64_t>(32, (32 << 20) / per / 2 * 2));
+        H->rx_entn = (int64_t)4 * g.nt + H->rx_T;
+        BZ_TRY(dalloc(&H->rx_pa, sizeof(bzk::PlanA<R, uint16_t>) * (size_t)K * g.nt));
+        BZ_TRY(dalloc(&H->rx_idx, sizeof(ushort4) * (size_t)K * g.nt));
+        BZ_TRY(dalloc(&H->rx_count, sizeof(int) * (size_t)K * g.nvt));
+        BZ_TRY(dalloc(&H->rx_cursor, sizeof(int) * (size_t)K * g.nvt));
+        BZ_TRY(dalloc(&H->rx_meta, sizeof(int) * 2 * K));
+        BZ_TRY(dalloc(&H->rx_ent, sizeof(uint32_t) * (size_t)K * H->rx_entn));
+        BZ_TRY(dalloc(&H->rx_cnt, sizeof(unsigned long long) * 2 * K));
+    }
+    H->relax = true;
+    return BZ_OK;
+}
+
+// The plans of steps [n, n + K) on stream s unless they cover [n, n + cnt)
+// (never while a stream is being captured).
+template <typename R>
+bz_status ensure_rx_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt)
+{
+    if (n >= H->rx_lo && n + cnt <= H->rx_hi) return BZ_OK;
+    const bzk::RxPlans<R> A = rx_plans<R>(H);
+    const int K = A.K;
+    ProfScope ps(H, 1, s);
+    BZ_CUDA(cudaMemsetAsync(A.cnt, 0, sizeof(unsigned long long) * 2 * K, s));
+    BZ_CUDA(cudaMemsetAsync(A.count, 0, sizeof(int) * (size_t)K * A.nvt, s));
+    bzk::k_rx_plan<R><<<dim3((A.nt + 63) / 64, K), 64, 0, s>>>(H->g, A, n);
+    BZ_LAUNCHED(H);
+    bzk::k_rx_scan<R><<<K, 1024, 0, s>>>(A);
+    BZ_LAUNCHED(H);
+    bzk::k_rx_fill<R><<<dim3((A.nt + 255) / 256, K), 256, 0, s>>>(A);
+    BZ_LAUNCHED(H);
+    H->rx_lo = n;
+    H->rx_hi = n + K;
+    return BZ_OK;
+}
+
+// The cells of one step from hin to hout, and the end of the step.
+template <typename R>
+bz_status launch_relax(bz_handle *H, cudaStream_t s, bool fused, const R *hin, R *hout)
+{
+    {
+        ProfScope ps(H, 2, s);
+        auto go = [&](auto *k) {
+            k<<<H->rx_grid, H->rx_T, H->rx_smem, s>>>(H->g, H->rx_nseg, hin, (const R *)H->ghost, rx_plans<R>(H), hout,
+                                                      H->mom, H->stats, H->d_step);
+        };
+        if (fused) with_relax_kernel<R, true>(H, go);
+        else with_relax_kernel<R, false>(H, go);
+        BZ_LAUNCHED(H);
+    }
+    H->cur ^= 1;
+    H->mom_valid = true;
+    if (H->per_cell) return advance(H, s);
+    bzk::k_rx_advance<<<1, 1, 0, s>>>(H->d_step, H->rx_K, H->rx_cnt, H->stats);
+    BZ_LAUNCHED(H);
+    H->step++;
+    return BZ_OK;
+}
+
 // One fused step on the active-node path: walls (applying the input's
 // pending corrections), the sample set, its compact form and scatter list,
 // the per-cell kernel, and the k_cell4 fallback that runs only when the step
@@ -703,6 +846,8 @@ bz_status configure_lazy(bz_handle *H)
 // a stream is being captured (the step graphs hold only k_ahead_take).
 bz_status ensure_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt)
 {
+    if (H->relax && !H->per_cell)
+        return H->dtype == BZ_F64 ? ensure_rx_plans<double>(H, s, n, cnt) : ensure_rx_plans<float>(H, s, n, cnt);
     if (!H->lazy || H->ahead_K == 0) return BZ_OK;
     if (n >= H->ahead_lo && n + cnt <= H->ahead_hi) return BZ_OK;
     const bzk::AheadPlans &A = H->ahead;
@@ -892,7 +1037,7 @@ bz_status launch_step(bz_handle *H, cudaStream_t s, bool fused, bool do_stream, 
     using V4 = typename bzk::Idx4<I>::type;
     using PA = bzk::PlanA<R, I>;
     if constexpr (sizeof(R) == 4) {
-        const bool ahead = H->ahead_K > 0;
+        const bool ahead = H->ahead_K > 0 && !H->captured;
         if (fused && H->lazy) return launch_lazy(H, s, true, false, ahead);
         // The relaxation alone on the active-node kernel (no streaming).
         if (!fused && do_collide && !do_stream && H->lazy) return launch_lazy(H, s, true, true, ahead);
@@ -908,7 +1053,9 @@ bz_status launch_step(bz_handle *H, cudaStream_t s, bool fused, bool do_stream, 
         bzk::k_walls<R><<<g.nfaces, bzk::kWallThreads, 0, s>>>(g, H->d_step, hin, (R *)H->ghost, H->nw, nullptr);
         BZ_LAUNCHED(H);
     }
-    if ((do_collide || fused) && !H->per_cell) {
+    const bool relax = H->relax && (H->per_cell || !H->captured);
+    if (fused && relax) return launch_relax<R>(H, s, true, hin, hout);
+    if ((do_collide || fused) && !H->per_cell && !relax) {
         ProfScope ps(H, 1, s);
         int pb = 256, pg = (g.nt + pb - 1) / pb;
         bzk::k_plan<R, I><<<pg, pb, 0, s>>>(g, H->d_step, (V4 *)H->pidx, (PA *)H->pa, nullptr, H->stats);
@@ -966,6 +1113,7 @@ bz_status launch_step(bz_handle *H, cudaStream_t s, bool fused, bool do_stream, 
         }
         hin = dst;
     }
+    if (do_collide && relax) return launch_relax<R>(H, s, false, hin, hout);
     if (do_collide && launch_cell4(H, s, false, hin, hout)) {
         BZ_LAUNCHED(H);
         H->cur ^= 1;
@@ -1081,6 +1229,9 @@ void release(bz_handle *H)
     void *ah[] = {A.idx, A.pa, A.qc, A.flag, A.cidx, A.act, A.mask, A.wpre, A.meta, A.count, A.cursor,
                   A.rowend, A.dest0, A.rec, A.cnt};
     for (void *p : ah)
+        if (p) cudaFree(p);
+    void *rx[] = {H->rx_pa, H->rx_idx, H->rx_count, H->rx_cursor, H->rx_meta, H->rx_ent, H->rx_cnt};
+    for (void *p : rx)
         if (p) cudaFree(p);
     bz_adj_release(&H->adj);
 }
@@ -1345,6 +1496,12 @@ bz_status bz_create(const bz_space *space, const bz_vel *vel, const bz_walls *wa
     g.lid_profile = walls->lid_profile ? H->profile : nullptr;
     st = configure_lazy(H);
     if (st != BZ_OK) return bail(st);
+    {
+        const char *force = getenv("BZ_KERNEL");
+        if (!H->lazy && !H->fast && H->idx16 && g.nt <= 65536 && !(force && strcmp(force, "generic") == 0))
+            st = H->dtype == BZ_F64 ? configure_relax<double>(H) : configure_relax<float>(H);
+        if (st != BZ_OK) return bail(st);
+    }
     *out = H;
     return BZ_OK;
 }
@@ -1484,12 +1641,18 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
         return fail(BZ_EINVAL, "unknown flags 0x%x", flags);
     if (fault_injected("launch")) return fail(BZ_ECUDA, "kernel launch failed (BZ_FAULT=launch)");
     cudaStream_t s = (cudaStream_t)stream;
+    // A graph that the caller captures may be replayed at any step: it holds
+    // the kernels that build each step's plan from the device step counter,
+    // not a batch of plans for the steps of the capture.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    H->captured = cap != cudaStreamCaptureStatusNone;
     bool fused = flags == 0;
     bool ds = (flags & BZ_DO_STREAM) || (flags & BZ_SPLIT);
     bool dc = (flags & BZ_DO_COLLIDE) || (flags & BZ_SPLIT);
     if (ds && dc && !H->ht) BZ_TRY(dalloc(&H->ht, H->esz * (size_t)H->g.nr * H->g.nvt));
     int32_t n = 0;
-    if (fused && nsteps >= 2 && graphs_enabled()) {
+    if (fused && nsteps >= 2 && graphs_enabled() && !H->captured) {
         // The captured steps read the buffers as they are now: bring the
         // pair into the state the steps leave it in before capturing.
         if (!H->lazy) {
@@ -1507,9 +1670,10 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
             if (H->lazy) H->lazy_buf[0] = H->lazy_buf[1] = true;
         }
     }
-    const bool planned = fused || (dc && !ds);   // the steps that run the active-node kernel
+    // The steps that run the active-node kernel or the cells with separate increments.
+    const bool planned = fused || (dc && (!ds || H->relax));
     for (; n < nsteps; ++n) {
-        if (planned) BZ_TRY(ensure_plans(H, s, H->step, 1));
+        if (planned && !H->captured) BZ_TRY(ensure_plans(H, s, H->step, 1));
         BZ_TRY(one_step(H, s, fused, ds, dc));
     }
     return BZ_OK;
