@@ -724,13 +724,17 @@ bzk::RxPlans<R> rx_plans(const bz_handle *H)
 }
 
 // Calls f with the k_relax instance of a handle.  FP64 has 512 threads at
-// most (32 sums of 8 bytes at the reduction), per-cell sets two CTAs of up to
-// 576 threads where two fit.
+// most (32 sums of 8 bytes at the reduction) and 128 registers, or 80 and a
+// third CTA per SM where there are more cells than the CTAs of the former
+// hold at once (33 x 47 x 14^3: ten steps 4158 -> 3885 us; 16^2 x 12^3, whose 256
+// cells fit at once, 668 -> 694); per-cell sets two CTAs of up to 576 threads
+// where two fit.
 template <typename R, bool FUSED, typename F>
 auto with_relax_kernel(const bz_handle *H, F f)
 {
     if constexpr (sizeof(R) == 8) {
-        return H->per_cell ? f(bzk::k_relax<double, FUSED, true, 512, 1>) : f(bzk::k_relax<double, FUSED, false, 512, 1>);
+        if (H->per_cell) return f(bzk::k_relax<double, FUSED, true, 512, 1>);
+        return H->rx_minb == 3 ? f(bzk::k_relax<double, FUSED, false, 256, 3>) : f(bzk::k_relax<double, FUSED, false, 512, 1>);
     } else {
         if (!H->per_cell) return f(bzk::k_relax<float, FUSED, false, 1024, 1>);
         return H->rx_minb == 2 ? f(bzk::k_relax<float, FUSED, true, 576, 2>) : f(bzk::k_relax<float, FUSED, true, 1024, 1>);
@@ -744,18 +748,17 @@ bz_status configure_relax(bz_handle *H)
     const int N = g.nv, N2 = N * N;
     const int maxt = sizeof(R) == 8 ? 512 : 1024;
     if (N2 > maxt) return BZ_OK;
-    // Segments of jx per column: to fill up to 512 threads where samples are
-    // drawn in the cell or FP32 does the sums; for FP64 (each segment repeats
-    // the 26 sums of its column) only where there are few cells per SM.
-    int nseg = 1;
-    if (H->per_cell || sizeof(R) == 4) nseg = std::max(1, 512 / N2);
-    else if (g.nr <= 4 * H->nsm) nseg = std::max(1, 448 / N2);
-    nseg = std::min(nseg, std::min(N, sizeof(R) == 8 ? 3 : 8));
+    // Segments of jx per column: to fill up to 512 threads in FP32.  FP64 is
+    // bound by its pipe, and each segment repeats the 26 sums of its column:
+    // one, and more CTAs per SM instead.
+    const int nseg = sizeof(R) == 8 ? 1 : std::min(std::max(1, 512 / N2), std::min(N, 8));
     H->rx_nseg = nseg;
     H->rx_T = (N2 * nseg + 31) / 32 * 32;
     H->rx_smem = bzk::rx_smem<R>(nullptr, nullptr, N, g.nvt, H->rx_T, H->per_cell ? 0 : g.nt);
     if (H->rx_smem > (size_t)H->smem_optin) return BZ_OK;
-    H->rx_minb = sizeof(R) == 4 && H->per_cell && H->rx_T <= 576 ? 2 : 1;
+    H->rx_minb = 1;
+    if (sizeof(R) == 4 && H->per_cell && H->rx_T <= 576) H->rx_minb = 2;
+    if (sizeof(R) == 8 && !H->per_cell && H->rx_T <= 256 && g.nr > H->nsm * (65536 / (128 * H->rx_T))) H->rx_minb = 3;
     int occ = 0;
     auto set = [&](auto *k) -> bz_status {
         int o = 0;

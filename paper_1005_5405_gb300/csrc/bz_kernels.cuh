@@ -213,13 +213,13 @@ __device__ __forceinline__ SampleOut draw_sample(const Geo &g, int64_t step, uin
 
 // The same sample in FP32, for FP32 states on uniform velocity grids.  The
 // coordinates that pick nodes are computed in FP32 with a bounded error: the
-// uniforms and k_z are rounded once from their integers, -ln u near u = 1
-// comes from the exact complement 1 - u, sin(theta) = 2 sqrt(u (1 - u)), and
-// the angles 2 pi u are split into a float part for sincospif and an exact
-// remainder added to first order.  With CUDA's 1-ulp bounds for logf, log1pf
-// and sincospif this keeps every coordinate of v and v1 within 1.3e-6 of its
-// exact value and every coordinate of v* and v1* within 2.4e-5 (|v| < 4.8 by
-// the Box-Muller radius at the smallest uniform).  A coordinate closer to a
+// uniforms and k_z are rounded once from their integers, -ln u takes the
+// rounding of u to first order, sin(theta) = 2 sqrt(u (1 - u)), and the angles
+// 2 pi u are split into a float part for sincospif and an exact remainder
+// added to first order.  With CUDA's 1-ulp bounds for logf and sincospif this
+// keeps every coordinate of v and v1 within 1.5e-6 of its exact value and
+// every coordinate of v* and v1* within 2.7e-5 (|v| < 4.8 by the Box-Muller
+// radius at the smallest uniform).  A coordinate closer to a
 // cell face than about four times its bound (kFastMarginA / kFastMarginB, in
 // velocity units, plus the rounding of the cell coordinate itself) sets
 // *redo: the caller draws that sample again with draw_sample.  Every other
@@ -233,11 +233,15 @@ __device__ __forceinline__ float u01f(uint32_t x)
 {
     return __fmaf_rn((float)(x & 255u) + 0.5f, 0x1p-32f, (float)(x >> 8) * 0x1p-24f);
 }
-// -ln u for u = (x + 1/2) 2^-32 (near u = 1 from 1 - u = (~x + 1/2) 2^-32).
+// -ln u for u = (x + 1/2) 2^-32: the logarithm of u rounded to float, uf, and
+// to first order the rounding error u - uf (exact; at most 2^-25, so that
+// 1/uf may be 2 - uf: within 2e-8 of the result, which is at least 0.69 where
+// that is off, and exact to 1e-8 of itself as u nears 1).
 __device__ __forceinline__ float neglog_u01f(uint32_t x)
 {
-    if (x < 0x80000000u) return -logf(u01f(x));
-    return -log1pf(-u01f(~x));
+    const float hi = (float)(x >> 8) * 0x1p-24f, lo = (float)(x & 255u) + 0.5f;
+    const float uf = __fmaf_rn(lo, 0x1p-32f, hi), du = __fmaf_rn(lo, 0x1p-32f, hi - uf);
+    return -__fmaf_rn(du, 2.f - uf, logf(uf));
 }
 // (sin, cos) of 2 pi u for u = (x + 1/2) 2^-32: with x read as a signed
 // integer the angle is pi t, t = (x + 1/2) 2^-31 in [-1, 1), split exactly
@@ -253,19 +257,20 @@ __device__ __forceinline__ void sincos_2pi_u01f(uint32_t x, float *sv, float *cv
     *sv = __fmaf_rn(c, d, s);
     *cv = __fmaf_rn(-s, d, c);
 }
-// Cell of one coordinate on a uniform axis (-1 outside the box); *near when
-// the coordinate lies within m cell widths of a face.
-__device__ __forceinline__ int node_axis_fast(float v, float vmax, float idv, int n, float m, bool *near)
+// Cell of one coordinate on a uniform axis (negative or >= n outside the box);
+// *near when the coordinate lies within m cell widths of a face.  t - 1/2 is
+// rounded to the nearest integer by adding 1.5 2^23 (|t| < 2^21); a tie or a
+// rounding the wrong way only happens next to a face.
+__device__ __forceinline__ int node_axis_fast(float v, float vmax, float idv, float m, bool *near)
 {
-    const float t = __fmul_rn(__fadd_rn(v, vmax), idv);
-    const float fl = floorf(t), fr = t - fl;
-    if (fr < m || fr > 1.f - m) *near = true;
-    if (!(t >= 0.f) || fl >= (float)n) return -1;
-    return (int)fl;
+    const float t = __fadd_rn(__fmul_rn(__fadd_rn(v, vmax), idv), -0.5f);
+    const float r = __fadd_rn(t, 12582912.f);
+    if (fabsf(__fsub_rn(t, __fsub_rn(r, 12582912.f))) > 0.5f - m) *near = true;
+    return __float_as_int(r) - 0x4B400000;
 }
 
 __device__ __forceinline__ SampleOut draw_sample_fast(const Geo &g, int64_t step, uint32_t cellword,
-                                                      uint32_t l, bool *redo)
+                                                      uint32_t l, bool *redo, float *Wf = nullptr)
 {
     const uint2 key = make_uint2(g.seed, g.instance);
     const uint4 a = philox4x32_10(make_uint4(l, (uint32_t)step, cellword, 0u), key);
@@ -290,10 +295,9 @@ __device__ __forceinline__ SampleOut draw_sample_fast(const Geo &g, int64_t step
     const int n = g.nv;
     bool near = false;
     auto node = [&](float x, float y, float z, float m) {
-        const int i = node_axis_fast(x, vmax, idv, n, m, &near),
-                  j = node_axis_fast(y, vmax, idv, n, m, &near),
-                  q = node_axis_fast(z, vmax, idv, n, m, &near);
-        return (i < 0 || j < 0 || q < 0) ? -1 : (i * n + j) * n + q;
+        const int i = node_axis_fast(x, vmax, idv, m, &near), j = node_axis_fast(y, vmax, idv, m, &near),
+                  q = node_axis_fast(z, vmax, idv, m, &near);
+        return max(max((uint32_t)i, (uint32_t)j), (uint32_t)q) >= (uint32_t)n ? -1 : (i * n + j) * n + q;
     };
     SampleOut o;
     o.idx[0] = node(v[0], v[1], v[2], ma);
@@ -303,7 +307,8 @@ __device__ __forceinline__ SampleOut draw_sample_fast(const Geo &g, int64_t step
     *redo = near;
     o.near = 0;
     o.outside = (o.idx[0] < 0) | (o.idx[1] < 0) | (o.idx[2] < 0) | (o.idx[3] < 0);
-    o.W = (double)(g.cwf * fabsf(s));
+    if (Wf) *Wf = g.cwf * fabsf(s);          // (no conversion to double and back)
+    else o.W = (double)(g.cwf * fabsf(s));
     return o;
 }
 

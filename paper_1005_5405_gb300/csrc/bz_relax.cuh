@@ -7,20 +7,20 @@
 // sample's product to it with four shared-memory atomics, and passes over it
 // again for the moments of N, of N_c and of the result.  Here h~ stays in its
 // slab and the increments dN = sum +-W g go to a second one, so that
-//   * the moments of h~ are summed while it is streamed (5 multiply-adds a
-//     node with tables of A v^k), and those of the increments from dN alone;
+//   * one pass forms h_c = h~ + dN / w where a sample reached the node and sums
+//     its moments (5 multiply-adds a node with tables of A v^k) and those of dN;
 //   * the output moments follow from the 30 sums of degree <= 4 and mu
 //     (lz_finish's formula), without a pass over the result;
 //   * a shared sample set is applied without atomics: each thread sums its run
 //     of the destination-sorted terms (k_scatter_*) in a register;
 //   * per-cell sets need no storage per sample (products and node indices),
 //     so two CTAs fit an SM where k_cell's 1024 threads had one.
-// FP64 work per node falls from about 25 operations to 12, plus 7 on nodes
+// FP64 work per node falls from about 25 operations to 12, plus 5 on nodes
 // that a sample reaches; GB300's FP64 pipe (about 2 a cycle and SM) bounds the
 // FP64 cells.  Ten steps with a
-// read-out, k_cell against k_relax: 16^2 x 12^3 FP64, 1000 samples, 1404 -> 980 us;
-// 33 x 47 x 14^3 FP64 stretched, 3000 samples, 6471 -> 4773 us; four steps of 64^2 x
-// 24^3 with 10^4 samples per cell (FP32) 10.74 -> 7.76 ms.
+// read-out, k_cell against k_relax: 16^2 x 12^3 FP64, 1000 samples, 1400 -> 668 us;
+// 33 x 47 x 14^3 FP64 stretched, 3000 samples, 6467 -> 3885 us; four steps of 64^2 x
+// 24^3 with 10^4 samples per cell (FP32) 10.73 -> 6.70 ms.
 #pragma once
 
 #include "bz_lazy.cuh"
@@ -32,8 +32,8 @@ constexpr int kRxMaxN = 32;
 template <typename R>
 struct RxSmem {
     R *Av;                  // [5][N]: A v^k
-    R *v, *IA, *cu, *ax, *cx;   // N each; ax: |Courant number| at the cell's width
-    R *E;                   // [5]: sum_j A v^k of one axis
+    R *v, *v2, *IA, *cu, *ax, *cx;  // N each; ax: |Courant number| at the cell's width
+    R *e0;                  // [32]: equilibrium sums of the 30 monomials
     R *part;                // [warps][32] partial sums; redraw queue of the per-cell sampler
     R *X, *D;               // [32] totals of N_c over the 30 monomials, [8] of dN
     R *mu;                  // [8]
@@ -52,11 +52,12 @@ __host__ __device__ inline size_t rx_smem(RxSmem<R> *s, char *base, int N, int n
     off = (off + 15) & ~(size_t)15;
     x.Av = take(5 * N);
     x.v = take(N);
+    x.v2 = take(N);
     x.IA = take(N);
     x.cu = take(N);
     x.ax = take(N);
     x.cx = take(N);
-    x.E = take(8);
+    x.e0 = take(32);
     x.part = take((size_t)(T / 32) * 32);
     x.X = take(32);
     x.D = take(8);
@@ -100,6 +101,10 @@ __device__ __forceinline__ void rx_mono(const R (&s)[5], R y, R z, R (&M)[32])
     M[24] = z * t3;
     M[25] = y * z * t2;
 }
+
+// A node that a sample reached (no FP64 comparison for doubles).
+__device__ __forceinline__ bool rx_set(float x) { return x != 0.f; }
+__device__ __forceinline__ bool rx_set(double x) { return __double_as_longlong(x) != 0; }
 
 // Sums of 32 values over a warp by recursive halving: lane l gets value l.
 template <typename R>
@@ -212,26 +217,12 @@ __device__ __forceinline__ void rx_finish(const Geo &g, const RxSmem<R> &S, doub
     const R eps = (R)g.eps;
     R m = R(0);
     if (lane < 10) {
-        // sum w h phi = sum N_c phi + sum_a mu_a (E0 + eps sum N_c psi_a phi),
-        // E0 of a monomial from the axis sums.
-        auto e0 = [&](int x) -> R {
-            const R *E = S.E;
-            constexpr unsigned char pw[26][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {2, 0, 0}, {0, 2, 0},
-                {0, 0, 2}, {1, 1, 0}, {1, 0, 1}, {0, 1, 1}, {3, 0, 0}, {0, 3, 0}, {0, 0, 3}, {2, 1, 0}, {2, 0, 1},
-                {1, 2, 0}, {0, 2, 1}, {1, 0, 2}, {0, 1, 2}, {1, 1, 1}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0},
-                {0, 0, 0}, {0, 0, 0}};
-            if (x < 20) return E[pw[x][0]] * E[pw[x][1]] * E[pw[x][2]];
-            const R e22 = E[2] * E[2] * E[0], e4 = E[4] * E[0] * E[0] + R(2) * e22;
-            if (x < 23) return e4;                       // v_i^2 v^2
-            if (x < 26) return R(2) * E[3] * E[1] * E[0] + E[1] * E[1] * E[2];
-            if (x == 26) return R(3) * E[2] * E[0] * E[0];
-            return E[3] * E[0] * E[0] + R(2) * E[1] * E[2] * E[0];
-        };
+        // sum w h phi = sum N_c phi + sum_a mu_a (E0 + eps sum N_c psi_a phi)
         m = X[lane];
 #pragma unroll 1
         for (int k = 0; k < 5; ++k) {
             const int x = S.px[k * 16 + lane];
-            m += S.mu[k] * (e0(x) + eps * X[x]);
+            m += S.mu[k] * (S.e0[x] + eps * X[x]);
         }
     }
     const unsigned all = 0xFFFFFFFFu;
@@ -352,19 +343,38 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
             x *= v;
         }
         S.v[i] = (R)v;
+        S.v2[i] = (R)(v * v);
         S.IA[i] = (R)(1.0 / A);
         S.cu[i] = (R)(v * g.dt / g.dx);
     }
-    if (t < 5) {
-        double s = 0.0;
-        for (int i = 0; i < N; ++i) {
-            double x = g.axA[i];
-            for (int k = 0; k < t; ++k) x *= g.axv[i];
-            s += x;
-        }
-        S.E[t] = (R)s;
+    if (t < 32) {
+        // The equilibrium sum of monomial t: a product of axis sums E_k = sum
+        // A v^k (lane k < 5 holds E_k), or for those with v^2 a sum of three.
+        double Ek = 0.0;
+        if (t < 5)
+            for (int i = 0; i < N; ++i) {
+                double x = g.axA[i];
+                for (int k = 0; k < t; ++k) x *= g.axv[i];
+                Ek += x;
+            }
+        double E[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) E[k] = __shfl_sync(0xFFFFFFFFu, Ek, k);
+        const double z = E[0], e22 = E[2] * E[2] * z, e31 = E[3] * E[1] * z, e112 = E[1] * E[1] * E[2];
+        double x = z * z * z;                                         // 1
+        if (t >= 1 && t <= 3) x = E[1] * z * z;                       // v_i
+        if (t >= 4 && t <= 6) x = E[2] * z * z;                       // v_i^2
+        if (t >= 7 && t <= 9) x = E[1] * E[1] * z;                    // v_i v_j
+        if (t >= 10 && t <= 12) x = E[3] * z * z;                     // v_i^3
+        if (t >= 13 && t <= 18) x = E[2] * E[1] * z;                  // v_i^2 v_j
+        if (t == 19) x = E[1] * E[1] * E[1];                          // v_x v_y v_z
+        if (t >= 20 && t <= 22) x = E[4] * z * z + 2.0 * e22;         // v_i^2 v^2
+        if (t >= 23 && t <= 25) x = 2.0 * e31 + e112;                 // v_i v_j v^2
+        if (t == 26) x = 3.0 * E[2] * z * z;                          // v^2
+        if (t >= 27) x = E[3] * z * z + 2.0 * E[1] * E[2] * z;        // v_i v^2
+        S.e0[t] = (R)x;
     }
-    if (t < 50) S.px[t / 10 * 16 + t % 10] = (unsigned char)lz_psiphi(t / 10, t % 10);
+    for (int i = t; i < 50; i += T) S.px[i / 10 * 16 + i % 10] = (unsigned char)lz_psiphi(i / 10, i % 10);
     // The thread's column and its range of jx.
     const bool col = t < N2 * nseg;
     const int seg = col ? t / N2 : 0, p = col ? t - seg * N2 : 0, jy = p / N, jz = p - jy * N;
@@ -383,8 +393,7 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
             for (int i = t; i < N; i += T) S.ax[i] = fabs(S.cu[i]) * fx;
             __syncthreads();
         }
-        // ---- h~, its power sums, and dN = 0
-        R s[5] = {R(0), R(0), R(0), R(0), R(0)};
+        // ---- h~, and dN = 0
         if (col) {
             R ay = R(0);
             const R *ys = own, *xr = own, *xl = own;
@@ -415,8 +424,6 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                 }
                 S.h[j] = h;
                 S.d[j] = R(0);
-#pragma unroll
-                for (int k = 0; k < 5; ++k) s[k] += S.Av[k * N + jx] * h;
             }
         }
         if (PC && t == 0) reinterpret_cast<int *>(S.part)[0] = 0;
@@ -428,9 +435,9 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
             int *rq = reinterpret_cast<int *>(S.part);
             const int room = (T / 32) * 32 * (int)(sizeof(R) / 4) - 1;
             const int rcap = g.redraw_cap < 0 ? room : min(g.redraw_cap, room);
-            auto put = [&](const SampleOut &o) {
+            auto put = [&](const SampleOut &o, R W) {
                 const R ha = o.idx[0] >= 0 ? S.h[o.idx[0]] : R(0), hb = o.idx[1] >= 0 ? S.h[o.idx[1]] : R(0);
-                const R r = (ha + hb + eps * ha * hb) * (R)o.W;
+                const R r = (ha + hb * (R(1) + eps * ha)) * W;
                 if (r == R(0)) return;
                 if (o.idx[2] >= 0) atomicAdd(S.d + o.idx[2], r);
                 if (o.idx[3] >= 0) atomicAdd(S.d + o.idx[3], r);
@@ -455,7 +462,8 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                 SampleOut o = {};
                 if (act) {
                     bool redo = true;
-                    if (fast) o = draw_sample_fast(g, step, (uint32_t)c, (uint32_t)l, &redo);
+                    float Wf = 0.f;
+                    if (fast) o = draw_sample_fast(g, step, (uint32_t)c, (uint32_t)l, &redo, &Wf);
                     if (redo) {
                         const int k = fast ? atomicAdd(rq, 1) : rcap;
                         if (k < rcap) {
@@ -465,7 +473,7 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                             o = draw_sample(g, step, (uint32_t)c, (uint32_t)l);
                         }
                     }
-                    if (act) put(o);
+                    if (act) put(o, redo ? (R)o.W : (R)Wf);
                 }
                 count(act, o);
             }
@@ -477,7 +485,7 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                     SampleOut o = {};
                     if (act) {
                         o = draw_sample(g, step, (uint32_t)c, (uint32_t)rq[1 + i0 + t]);
-                        put(o);
+                        put(o, (R)o.W);
                     }
                     count(act, o);
                 }
@@ -487,7 +495,7 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                 const PlanA<R, uint16_t> q = pa[l];
                 const int a = q.a(), b = q.b();
                 const R ha = a >= 0 ? S.h[a] : R(0), hb = b >= 0 ? S.h[b] : R(0);
-                S.gw[l] = (ha + hb + eps * ha * hb) * q.W;
+                S.gw[l] = (ha + hb * (R(1) + eps * ha)) * q.W;
             }
             __syncthreads();
             // Each thread's run of the sorted terms: a destination's sum is
@@ -523,31 +531,35 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
         }
         __syncthreads();
 
-        // ---- sums of dN and of N_c over the monomials, the correction
+        // ---- h_c = h~ + dN / w, the sums of dN and of N_c = w h_c, the correction
         R M[32];
         {
-            R d[5] = {R(0), R(0), R(0), R(0), R(0)};
+            R s[5] = {R(0), R(0), R(0), R(0), R(0)}, d0 = R(0), d1 = R(0), d2 = R(0);
             if (col) {
+#pragma unroll 2
                 for (int jx = x0; jx < x1; ++jx) {
-                    const R x = S.d[jx * N2 + p];
-                    if (x != R(0)) {
-                        const R v = S.v[jx], v2 = v * v;
-                        d[0] += x;
-                        d[1] += x * v;
-                        d[2] += x * v2;
-                        d[3] += x * (v2 * v);
-                        d[4] += x * (v2 * v2);
+                    const int j = jx * N2 + p;
+                    const R x = S.d[j];
+                    R h = S.h[j];
+                    if (rx_set(x)) {
+                        h += (x * IAyz) * S.IA[jx];
+                        S.h[j] = h;
+                        d0 += x;
+                        d1 += x * S.v[jx];
+                        d2 += x * S.v2[jx];
                     }
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) s[k] += S.Av[k * N + jx] * h;
                 }
 #pragma unroll
-                for (int k = 0; k < 5; ++k) s[k] = s[k] * Ayz + d[k];
+                for (int k = 0; k < 5; ++k) s[k] *= Ayz;
             }
             rx_mono(s, vy, vz, M);
-            M[26] = d[0];
-            M[27] = d[1];
-            M[28] = vy * d[0];
-            M[29] = vz * d[0];
-            M[30] = d[2] + (vy * vy + vz * vz) * d[0];
+            M[26] = d0;
+            M[27] = d1;
+            M[28] = vy * d0;
+            M[29] = vz * d0;
+            M[30] = d2 + (vy * vy + vz * vz) * d0;
             M[31] = R(0);
         }
         S.part[warp * 32 + lane] = rx_reduce_scatter(M);
@@ -574,17 +586,15 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
         }
         __syncthreads();
 
-        // ---- h_c = h~ + dN / w, corrected
+        // ---- the corrected result
         if (col) {
             const R ct = S.mu[0] + S.mu[2] * vy + S.mu[3] * vz + S.mu[4] * (vy * vy + vz * vz);
             R *dst = hout + (int64_t)c * nvt;
 #pragma unroll 4
             for (int jx = x0; jx < x1; ++jx) {
                 const int j = jx * N2 + p;
-                const R x = S.d[j];
-                R h = S.h[j];
-                if (x != R(0)) h += x * (S.IA[jx] * IAyz);
-                dst[j] = h + (R(1) + eps * h) * (ct + S.cx[jx]);
+                const R h = S.h[j], kap = ct + S.cx[jx];
+                dst[j] = h + (R(1) + eps * h) * kap;
             }
         }
         __syncthreads();
