@@ -7,7 +7,7 @@
 #include "bz.h"
 #include "bz_internal.h"
 #include "bz_adjoint.cuh"
-#include "bz_cell4.cuh"
+#include "bz_adjcell4.cuh"
 
 #include <cuda_runtime.h>
 
@@ -95,7 +95,7 @@ bz_status prepare_fast(bz_adj_scratch *a, const bzk::Geo &g, int nsm, int optin)
     const int N = g.nv, Q = N * N / 4;
     const char *force = getenv("BZ_KERNEL");
     if (force && std::string(force) == "generic") return BZ_OK;
-    if (N % 4 != 0 || N < 12 || g.nvt >= 65535 || g.nt > 32768 || Q > 1024) return BZ_OK;
+    if (N % 4 != 0 || N < 12 || g.nvt >= 16384 || g.nt > 32768 || Q > 1024) return BZ_OK;
     const size_t smem = bzk::adj4_smem_bytes(N, g.nvt, g.nt);
     if (smem > (size_t)optin) return BZ_OK;
     // Two CTAs of up to 512 threads per SM when their shared memory fits, so
@@ -122,8 +122,8 @@ bz_status prepare_fast(bz_adj_scratch *a, const bzk::Geo &g, int nsm, int optin)
                              sizeof(int) * 2 * (size_t)g.nvt,
                              sizeof(int) * 2 * (size_t)g.nvt,
                              sizeof(int) * 4,
-                             sizeof(uint32_t) * ((size_t)4 * g.nt + bzk::kMaxThreads),
-                             sizeof(uint4) * ((size_t)2 * g.nt + bzk::kMaxThreads)};
+                             sizeof(uint32_t) * ((size_t)4 * g.nt + 4 * bzk::kMaxThreads),
+                             sizeof(uint2) * ((size_t)2 * g.nt + 2 * bzk::kMaxThreads)};
     void **dst[7] = {&a->pidx16, &a->pa16, (void **)&a->sc_count, (void **)&a->sc_cursor,
                      (void **)&a->sc_meta, (void **)&a->sc_ent, (void **)&a->lrec};
     void **dstb[7] = {&a->pidx16b, &a->pa16b, (void **)&a->sc_countb, (void **)&a->sc_cursorb,
@@ -151,7 +151,7 @@ bz_status prepare_fast(bz_adj_scratch *a, const bzk::Geo &g, int nsm, int optin)
 // forward and loss lists, as the forward step builds them (64-thread blocks
 // spread the FP64 sampling over every SM).
 cudaError_t fast_plan(const bzk::Geo &g, const int64_t *stepp, int threads, void *pidx16, void *pa16,
-                      int *sc_count, int *sc_cursor, int *sc_meta, uint32_t *sc_ent, uint4 *lrec,
+                      int *sc_count, int *sc_cursor, int *sc_meta, uint32_t *sc_ent, uint2 *lrec,
                       cudaStream_t sp, int *n)
 {
     bzk::Geo gs = g;
@@ -166,8 +166,8 @@ cudaError_t fast_plan(const bzk::Geo &g, const int64_t *stepp, int threads, void
     if (e != cudaSuccess) return e;
     bzk::k_adj_count2<<<pg, pb, 0, sp>>>(g.nt, g.nvt, pi, sc_count);
     bzk::k_adj_scan2<<<2, 1024, 0, sp>>>(g.nvt, threads, sc_count, sc_cursor, sc_meta);
-    bzk::k_adj_fill2<<<pg, pb, 0, sp>>>(g.nt, g.nvt, threads, pi, (const bzk::PlanA<float, uint16_t> *)pa16,
-                                        sc_cursor, sc_meta, sc_ent, lrec);
+    bzk::k_adj_fill2<<<pg, pb, 0, sp>>>(g.nt, g.nvt, threads, (ushort4 *)pidx16,
+                                        (bzk::PlanA<float, uint16_t> *)pa16, sc_cursor, sc_meta, sc_ent, lrec);
     *n += 3;
     return cudaGetLastError();
 }
@@ -186,7 +186,6 @@ bz_status launch(bz_adj_scratch *a, const bzk::Geo &g0, int64_t step, const R *h
     };
     bzk::k_set_step<<<1, 1, 0, s>>>(a->step, step);
     cudaError_t e = check();
-    const int pb = 256, pg = (g.nt + pb - 1) / pb;
     bool fast = false;
     if constexpr (sizeof(R) == 4) fast = a->fast;
     // The fast path's plan depends on the step only: it runs on the side
@@ -216,21 +215,15 @@ bz_status launch(bz_adj_scratch *a, const bzk::Geo &g0, int64_t step, const R *h
     }
     if (fast && e == cudaSuccess) e = cudaStreamWaitEvent(s, a->join, 0);
     if (fast) {
-        const ushort4 *pi = (const ushort4 *)a->pidx16;
         bzk::Geo gs = g;
         gs.swz = 1;
         if (e == cudaSuccess) {
             const bzk::Map4 m{a->map[0], a->map[1], a->map[2]};
-            if (a->threads <= 512)
-                bzk::k_adj_cell4<512><<<a->grid, a->threads, a->smem, s>>>(
-                    gs, m, (const float *)hn, (const float *)a->ghost, pi,
-                    (const bzk::PlanA<float, uint16_t> *)a->pa16, a->sc_ent, a->sc_meta, a->lrec,
-                    a->sc_meta + 2, (const float *)lam_in, (float *)a->lt, stats);
-            else
-                bzk::k_adj_cell4<1024><<<a->grid, a->threads, a->smem, s>>>(
-                    gs, m, (const float *)hn, (const float *)a->ghost, pi,
-                    (const bzk::PlanA<float, uint16_t> *)a->pa16, a->sc_ent, a->sc_meta, a->lrec,
-                    a->sc_meta + 2, (const float *)lam_in, (float *)a->lt, stats);
+            const auto kern = a->threads <= 512 ? bzk::k_adj_cell4<512> : bzk::k_adj_cell4<1024>;
+            kern<<<a->grid, a->threads, a->smem, s>>>(
+                gs, m, (const float *)hn, (const float *)a->ghost, (const uint2 *)a->pidx16,
+                (const uint2 *)a->pa16, (const uint4 *)a->sc_ent, a->sc_meta, (const uint4 *)a->lrec, (const float *)lam_in,
+                (float *)a->lt, stats);
             e = check();
         }
         // The plan of the step the next call is expected to take, into the

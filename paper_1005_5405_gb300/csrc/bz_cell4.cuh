@@ -412,294 +412,7 @@ __device__ __forceinline__ void cell4_setup(const Geo &g, const Cell4Smem &S)
 // One cell c of instance g: streaming into the slab (FUSED) or a copy of
 // h~, the Monte Carlo gather and scatter, the correction and the write-back.
 // Called by every thread of the CTA with the tables of g in place.
-// What the adjoint mode of cell4_cell adds: two more slabs (N_c, then
-// lam_c / w; dJ/dh~), 20 saved correction sums, a per-jx table, lam of the
-// cell in and dJ/dh~ out (global, logical order), the sample set.
-struct Adj4 {
-    float4 *B, *C;
-    float *P, *cxi;
-    const float *lam;
-    float *lt;
-    const ushort4 *pidx;
-    // The loss terms of the step (destination a or b of a sample), sorted by
-    // destination in runs of lmeta[1] records per thread (k_adj_fill2);
-    // lmeta[0] is their number.
-    const uint4 *lrec;
-    const int *lmeta;
-};
-
-// The adjoint's two lists of the step's terms.  The forward list: every
-// (node, sample, sign) term, as for k_cell4 (k_scatter_fill).  The loss
-// list of the transposed update: per sample with nodes (a, b, a*, b*) in the
-// shared-memory order (0xFFFF outside the grid) and weight W, one record for
-// each valid destination d in {a, b}:
-//   {a* | b* << 16, a | b << 16, W, d | (d is b) << 16}.
-// Counts, cursors and headers of the forward list come first, those of the
-// loss list nvt entries (two ints) after them.
-static __global__ void k_adj_count2(int nt, int nvt, const ushort4 *__restrict__ pidx,
-                                    int *__restrict__ count)
-{
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= nt) return;
-    const ushort4 q = pidx[l];
-    if (q.x != 0xFFFF) {
-        atomicAdd(count + q.x, 1);
-        atomicAdd(count + nvt + q.x, 1);
-    }
-    if (q.y != 0xFFFF) {
-        atomicAdd(count + q.y, 1);
-        atomicAdd(count + nvt + q.y, 1);
-    }
-    if (q.z != 0xFFFF) atomicAdd(count + q.z, 1);
-    if (q.w != 0xFFFF) atomicAdd(count + q.w, 1);
-}
-static __global__ void __launch_bounds__(1024) k_adj_scan2(int nvt, int T, const int *__restrict__ count,
-                                                           int *__restrict__ cursor, int *__restrict__ meta)
-{
-    __shared__ int part[1024];
-    const int k = blockIdx.x;
-    scatter_scan_body(nvt, T, count + k * nvt, cursor + k * nvt, meta + 2 * k, part);
-}
-static __global__ void k_adj_fill2(int nt, int nvt, int T, const ushort4 *__restrict__ pidx,
-                                   const PlanA<float, uint16_t> *__restrict__ pa,
-                                   int *__restrict__ cursor, const int *__restrict__ meta,
-                                   uint32_t *__restrict__ ent, uint4 *__restrict__ rec)
-{
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= nt) return;
-    const ushort4 q = pidx[l];
-    const unsigned short d[4] = {q.x, q.y, q.z, q.w};
-    const int C = meta[1], CL = meta[3];
-    const uint32_t gain = (uint32_t)q.z | ((uint32_t)q.w << 16), loss = (uint32_t)q.x | ((uint32_t)q.y << 16);
-    const uint32_t W = __float_as_uint(pa[l].W);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (d[k] == 0xFFFF) continue;
-        const int pos = atomicAdd(cursor + d[k], 1), tt = pos / C, i = pos - tt * C;
-        ent[(int64_t)i * T + tt] = ((uint32_t)d[k] << 16) | (k < 2 ? 0x8000u : 0u) | (uint32_t)l;
-        if (k < 2) {
-            const int pl = atomicAdd(cursor + nvt + d[k], 1), tl = pl / CL, il = pl - tl * CL;
-            rec[(int64_t)il * T + tl] = make_uint4(gain, loss, W, (uint32_t)d[k] | ((uint32_t)k << 16));
-        }
-    }
-}
-
-// x = G^{-1} rhs for the Gram matrix G = G0 + eps sum_j N_c,j psi_j psi_j^T
-// of the correction (P[0..13] its moment sums, as in correction_spd), by
-// elimination without pivoting (in registers; stable for the symmetric
-// positive definite G); Cholesky, then pivoted elimination, if a pivot is not
-// positive (fallback counted).
-static __device__ __noinline__ void gram_solve(const Geo &g, const float *P, const float *rhs, float *x,
-                                        int *fallback)
-{
-    const float e = g.epsf;
-    const float p4 = P[4] + P[5] + P[6];
-    const float m[5][5] = {
-        {P[0], P[1], P[2], P[3], p4},
-        {P[1], P[4], P[7], P[8], P[10]},
-        {P[2], P[7], P[5], P[9], P[11]},
-        {P[3], P[8], P[9], P[6], P[12]},
-        {p4, P[10], P[11], P[12], P[13]}};
-    float G[5][5], U[5][5], b[5], y[5];
-    bool ok = !g.solve_fb;
-#pragma unroll
-    for (int a = 0; a < 5; ++a) {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) G[a][c] = U[a][c] = g.G0f[a * 5 + c] + e * m[a][c];
-        b[a] = y[a] = rhs[a];
-    }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        ok = ok && U[k][k] > 0.f;
-        const float ip = 1.f / U[k][k];
-#pragma unroll
-        for (int i = k + 1; i < 5; ++i) {
-            const float f = U[i][k] * ip;
-#pragma unroll
-            for (int j = k + 1; j < 5; ++j) U[i][j] -= f * U[k][j];
-            y[i] -= f * y[k];
-        }
-    }
-    if (ok) {
-#pragma unroll
-        for (int i = 4; i >= 0; --i) {
-            float s = y[i];
-#pragma unroll
-            for (int j = i + 1; j < 5; ++j) s -= U[i][j] * x[j];
-            x[i] = s / U[i][i];
-        }
-        return;
-    }
-    chol_or_ge<float>(G, b, x, fallback, g.solve_fb != 0);
-}
-
-// Adjoint part of one cell (after the forward recompute of cell4_cell in
-// adjoint mode: S.slab4 holds h~, X.B holds N_c, muf[0..4] mu, X.P the sums
-// of G).  With lam = dJ/dh^{n+1} of the cell:
-//   nu = sum_j lam_j (1 + eps h_c,j) psi_j,  xi = G^{-1} nu,
-//   lam_c,j = (lam_j - w_j psi_j.xi)(1 + eps psi_j.mu)      (dJ/dN_c times w)
-//   dJ/dh~_j = lam_c,j + w_j psi_j.xi                        (N = w h~ and pre)
-//   gamma_l = W_l (q_a* + q_b* - q_a - q_b),  q = lam_c / w  (dJ/d(g_l W_l))
-//   dJ/dh~_a += gamma_l (1 + eps h~_b),  dJ/dh~_b += gamma_l (1 + eps h~_a).
-__device__ __forceinline__ void adj4_tail(const Geo &g, const Map4 &m, int c, const Cell4Smem &S,
-                                          const Adj4 &X, const PlanA<float, uint16_t> *__restrict__ pa,
-                                          float *muf, int &fallback)
-{
-    const int N = g.nv, nvt = g.nvt, T = blockDim.x, t = threadIdx.x;
-    const float eps = g.epsf;
-    float *totf = reinterpret_cast<float *>(S.tot);
-    const int Q = m.Q, nq = N / 4, q = t % Q, kchunk = t / Q;
-    const bool active = kchunk < m.K;
-    const int jy = q / nq, qz = q % nq, rowq = jy * nq;
-    const int jx0 = active ? kchunk * m.J : 0, jx1 = active ? jx0 + m.J : 0;
-    auto phys = [&](int jx) {
-        int r = qz + S.rot[jx];
-        r -= r >= nq ? nq : 0;
-        return jx * Q + rowq + r;
-    };
-    const float vy = S.v[jy];
-
-    // ---- nu, with lam of the cell staged into C ----------------------------
-    float nu[5];
-    {
-        float a0 = 0.f, a1 = 0.f, a3 = 0.f, a4 = 0.f;
-        if (active) {
-            const float4 *lam4 = reinterpret_cast<const float4 *>(X.lam + (int64_t)c * nvt);
-            const float4 z4 = S.vzq[qz], i4 = S.IAzq[qz];
-            const float iay = S.IA[jy];
-            const float vz[4] = {z4.x, z4.y, z4.z, z4.w};
-            const float IAyz[4] = {iay * i4.x, iay * i4.y, iay * i4.z, iay * i4.w};
-            float qq[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) qq[i] = vy * vy + vz[i] * vz[i];
-#pragma unroll 2
-            for (int jx = jx0; jx < jx1; ++jx) {
-                const int o = phys(jx);
-                const float4 n = X.B[o], l = lam4[jx * Q + q];
-                X.C[o] = l;
-                const float4 gv = S.gram[jx];      // v, v^2, v^3, v^4
-                const float ia = S.IA[jx];
-                const float nn[4] = {n.x, n.y, n.z, n.w}, ll[4] = {l.x, l.y, l.z, l.w};
-                float ts = 0.f, tz = 0.f, tq = 0.f;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float hc = nn[i] * (ia * IAyz[i]);
-                    const float tv = ll[i] * (1.f + eps * hc);
-                    ts += tv;
-                    tz += tv * vz[i];
-                    tq += tv * qq[i];
-                }
-                a0 += ts;
-                a1 += ts * gv.x;
-                a3 += tz;
-                a4 += ts * gv.y + tq;
-            }
-        }
-        nu[0] = a0;
-        nu[1] = a1;
-        nu[2] = vy * a0;
-        nu[3] = a3;
-        nu[4] = a4;
-    }
-    block_reduce4<5>(nu, S.red, totf);
-    float *xif = muf + 8;
-    if (t == 0) gram_solve(g, X.P, totf, xif, &fallback);
-    __syncthreads();
-    for (int i = t; i < N; i += T) X.cxi[i] = xif[1] * S.v[i] + xif[4] * S.v[i] * S.v[i];
-    __syncthreads();
-
-    // ---- lam_c / w into B, lam_c + w psi.xi into C ---------------------------
-    if (active) {
-        const float4 z4 = S.vzq[qz], a4v = S.Azq[qz], i4 = S.IAzq[qz];
-        const float ay = S.A[jy], iay = S.IA[jy];
-        const float vz[4] = {z4.x, z4.y, z4.z, z4.w};
-        const float Ayz[4] = {ay * a4v.x, ay * a4v.y, ay * a4v.z, ay * a4v.w};
-        const float IAyz[4] = {iay * i4.x, iay * i4.y, iay * i4.z, iay * i4.w};
-        float ctm[4], cti[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float qi = vy * vy + vz[i] * vz[i];
-            ctm[i] = muf[0] + muf[2] * vy + muf[3] * vz[i] + muf[4] * qi;
-            cti[i] = xif[0] + xif[2] * vy + xif[3] * vz[i] + xif[4] * qi;
-        }
-#pragma unroll 2
-        for (int jx = jx0; jx < jx1; ++jx) {
-            const int o = phys(jx);
-            const float4 l = X.C[o];
-            const float4 fv = S.fin[jx];          // 1/A, cx, A, A v
-            const float cxi = X.cxi[jx];
-            const float ll[4] = {l.x, l.y, l.z, l.w};
-            float bq[4], cq[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float w = fv.z * Ayz[i], px = cti[i] + cxi, pm = ctm[i] + fv.y;
-                const float lc = (ll[i] - w * px) * (1.f + eps * pm);
-                bq[i] = lc * (fv.x * IAyz[i]);
-                cq[i] = lc + w * px;
-            }
-            X.B[o] = make_float4(bq[0], bq[1], bq[2], bq[3]);
-            X.C[o] = make_float4(cq[0], cq[1], cq[2], cq[3]);
-        }
-    }
-    __syncthreads();
-
-    // ---- transposed Monte Carlo update --------------------------------------
-    // Each thread walks its run of the destination-sorted loss terms: the
-    // term of sample l at its node d in {a, b} adds gamma_l (1 + eps h~_p),
-    // p the other pre-collision node, to dJ/dh~_d.  A destination's sum is
-    // added plainly once the run leaves it, atomically for the run's first
-    // and last destinations (neighbouring runs may share them).
-    {
-        const float *Bf = reinterpret_cast<const float *>(X.B);
-        const float *Af = reinterpret_cast<const float *>(S.slab4);
-        float *Cf = reinterpret_cast<float *>(X.C);
-        const int E = X.lmeta[0], C = X.lmeta[1];
-        const int n = max(0, min(C, E - t * C));
-        int cur = -1;
-        bool first = true;
-        float acc = 0.f;
-        auto qv = [&](uint32_t i) { return i != 0xFFFFu ? Bf[i] : 0.f; };
-        auto term = [&](uint4 r) {
-            const float gam = __uint_as_float(r.z) * ((qv(r.x & 0xFFFFu) + qv(r.x >> 16)) -
-                                                      (qv(r.y & 0xFFFFu) + qv(r.y >> 16)));
-            const uint32_t p = (r.w >> 16) ? (r.y & 0xFFFFu) : (r.y >> 16);
-            const float hp = p != 0xFFFFu ? Af[p] : 0.f;
-            const int d = (int)(r.w & 0xFFFFu);
-            if (d != cur) {
-                if (cur >= 0) {
-                    if (first) atomicAdd(Cf + cur, acc);
-                    else Cf[cur] += acc;
-                    first = false;
-                }
-                cur = d;
-                acc = 0.f;
-            }
-            acc = fmaf(gam, fmaf(eps, hp, 1.f), acc);
-        };
-        const uint4 *rp = X.lrec + t;
-        int i = 0;
-        for (; i + 3 < n; i += 4) {
-            uint4 r[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) r[u] = rp[(int64_t)(i + u) * T];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) term(r[u]);
-        }
-        for (; i < n; ++i) term(rp[(int64_t)i * T]);
-        if (cur >= 0) atomicAdd(Cf + cur, acc);
-    }
-    __syncthreads();
-
-    // ---- dJ/dh~ of the cell out (logical order) ------------------------------
-    if (active) {
-        float4 *dst = reinterpret_cast<float4 *>(X.lt + (int64_t)c * nvt);
-#pragma unroll 2
-        for (int jx = jx0; jx < jx1; ++jx) dst[jx * Q + q] = X.C[phys(jx)];
-    }
-    __syncthreads();
-}
-
-template <bool FUSED, bool ADJ = false>
+template <bool FUSED>
 __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
                                            const float *__restrict__ hin,
                                            const float *__restrict__ ghost,
@@ -707,12 +420,8 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
                                            const uint32_t *__restrict__ ent,
                                            const int *__restrict__ meta, float *__restrict__ hout,
                                            double *__restrict__ mom, const Cell4Smem &S,
-                                           int &fallback, long long *__restrict__ clk, int ncell,
-                                           const Adj4 *X = nullptr)
+                                           int &fallback, long long *__restrict__ clk, int ncell)
 {
-    // The forward step works in place on one slab; the adjoint keeps h~ in
-    // the slab and builds N, N_c in a second one.
-    float4 *nsl = ADJ ? X->B : S.slab4;
     const int N = g.nv, nvt = g.nvt, T = blockDim.x, t = threadIdx.x;
     auto stamp = [&](int ph) {
         if (clk && blockIdx.x == 0 && t == 0 && ncell < kClkCells)
@@ -864,7 +573,7 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
             const float4 cv = S.conv[jx];        // {A, v, v^2, -}
             float n0 = h.x * (cv.x * Ayz[0]), n1 = h.y * (cv.x * Ayz[1]);
             float n2 = h.z * (cv.x * Ayz[2]), n3 = h.w * (cv.x * Ayz[3]);
-            nsl[o] = make_float4(n0, n1, n2, n3);
+            S.slab4[o] = make_float4(n0, n1, n2, n3);
             const float sn = (n0 + n1) + (n2 + n3);
             p0 += sn;
             p1 += sn * cv.y;
@@ -880,7 +589,7 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
     // Each thread walks its run of the destination-sorted list, sums the
     // terms of one node in a register and adds the sum with one atomic.
     {
-        float *slabw = reinterpret_cast<float *>(nsl);
+        float *slabw = reinterpret_cast<float *>(S.slab4);
         const int E = meta[0], C = meta[1];
         const int base = t * C, n = max(0, min(C, E - base));
         // Only the first and the last node of a run can be shared with the
@@ -936,7 +645,7 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
         if (active) {
 #pragma unroll 2
             for (int jx = jx0; jx < jx1; ++jx) {
-                float4 n = nsl[phys(jx)];
+                float4 n = S.slab4[phys(jx)];
                 const float4 gv = S.gram[jx];   // v, v^2, v^3, v^4
                 const float nn[4] = {n.x, n.y, n.z, n.w};
 #pragma unroll
@@ -998,8 +707,6 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
                 ++fallback;
                 for (int a = 0; a < 5; ++a) muf[a] = (float)m8[a];
             }
-            if constexpr (ADJ)
-                for (int a = 0; a < 14; ++a) X->P[a] = totf[a];
         }
     }
     __syncthreads();
@@ -1007,11 +714,6 @@ __device__ __forceinline__ void cell4_cell(const Geo &g, const Map4 &m, int c,
     for (int i = t; i < N; i += T) S.fin[i].y = mux * S.v[i] + mu4 * S.v[i] * S.v[i];
     __syncthreads();
     stamp(6);
-
-    if constexpr (ADJ) {
-        adj4_tail(g, m, c, S, *X, pa, muf, fallback);
-        return;
-    }
 
     // ---- corrected write-back and output moments ---------------------------
     float mo[10];
@@ -1086,133 +788,6 @@ k_cell4(Geo g, Map4 m, const float *__restrict__ hin, const float *__restrict__ 
     for (int kc = blockIdx.x; kc < g.nr; kc += gridDim.x, ++ncell)
         cell4_cell<FUSED>(g, m, cell_of(g, kc), hin, ghost, pa, ent, meta, hout, mom, S,
                           fallback, clk, ncell);
-    if (fallback && stats) atomicAdd(stats + 3, (unsigned long long)fallback);
-}
-
-
-// dJ/dh^n from dJ/dh~ (FP32, velocity axis a multiple of 4): the transposed
-// upwind stencil (h^n_c feeds h~ of its downwind neighbours: right for v_x >
-// 0, above for v_y > 0) in 16-byte quads of four jz nodes, plus on boundary
-// cells the outgoing-flux terms lF[f] |v_n| w of their faces and on the lid
-// row the lid-shear term wD 2 w v_x v_y / nx.  blockDim a multiple of Q.
-static __global__ void __launch_bounds__(1024) k_adj_stream4(Geo g, const float *__restrict__ lt,
-                                                             const double *__restrict__ lF,
-                                                             float *__restrict__ lam_out, double wD)
-{
-    __shared__ float sv[kMaxN], sax[kMaxN], say[kMaxN], sA[kMaxN];
-    const int N = g.nv, nq = N / 4, Q = N * N / 4, half = N / 2;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const double v = g.axv[i];
-        sv[i] = (float)v;
-        sax[i] = (float)(fabs(v) * g.dt / g.dx);
-        say[i] = (float)(fabs(v) * g.dt / g.dy);
-        sA[i] = (float)g.axA[i];
-    }
-    __syncthreads();
-    const int64_t plane = g.nvt / 4;
-    const int q = threadIdx.x % Q, jxs = threadIdx.x / Q, jstep = blockDim.x / Q;
-    const int jy = q / nq, jz0 = 4 * (q % nq);
-    const float vy = sv[jy], ay = say[jy];
-    const float dcoef = (float)(wD * 2.0 / g.nx);
-    for (int kc = blockIdx.x; kc < g.nr; kc += gridDim.x) {
-        const int c = cell_of(g, kc);
-        const int ix = c % g.nx, iy = c / g.nx;
-        const float4 *own = reinterpret_cast<const float4 *>(lt) + (int64_t)c * plane;
-        float4 *dst = reinterpret_cast<float4 *>(lam_out) + (int64_t)c * plane;
-        // Downwind y neighbour of this thread's row (v_y > 0: above).
-        const float4 *ys = own + (jy >= half ? (int64_t)g.nx : -(int64_t)g.nx) * plane;
-        if (ix > 0 && ix < g.nx - 1 && iy > 0 && iy < g.ny - 1) {
-            // Interior cell: both downwind neighbours are cells.
-            const float4 *xr = own + plane, *xl = own - plane;
-#pragma unroll 4
-            for (int jx = jxs; jx < N; jx += jstep) {
-                const int o = jx * Q + q;
-                const float ax = sax[jx];
-                const float4 l0 = own[o], lx = jx >= half ? xr[o] : xl[o], ly = ys[o];
-                const float c0 = 1.f - ax - ay;
-                dst[o] = make_float4(c0 * l0.x + ax * lx.x + ay * ly.x, c0 * l0.y + ax * lx.y + ay * ly.y,
-                                     c0 * l0.z + ax * lx.z + ay * ly.z, c0 * l0.w + ax * lx.w + ay * ly.w);
-            }
-            continue;
-        }
-        const bool yd = jy >= half ? iy < g.ny - 1 : iy > 0;
-        for (int jx = jxs; jx < N; jx += jstep) {
-            const int o = jx * Q + q;
-            const float ax = sax[jx];
-            const bool xd = jx >= half ? ix < g.nx - 1 : ix > 0;   // v_x > 0: right
-            const float4 l0 = own[o];
-            const float4 lx = xd ? own[o + (jx >= half ? plane : -plane)] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 ly = yd ? ys[o] : make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 r;
-            const float c0 = 1.f - ax - ay;
-            r.x = c0 * l0.x + ax * lx.x + ay * ly.x;
-            r.y = c0 * l0.y + ax * lx.y + ay * ly.y;
-            r.z = c0 * l0.z + ax * lx.z + ay * ly.z;
-            r.w = c0 * l0.w + ax * lx.w + ay * ly.w;
-            const float vx = sv[jx];
-            float ex = 0.f;
-            if (ix == 0 && vx < 0.f) ex -= (float)lF[iy] * vx;
-            if (ix == g.nx - 1 && vx > 0.f) ex += (float)lF[g.ny + iy] * vx;
-            if (iy == 0 && vy < 0.f) ex -= (float)lF[2 * g.ny + ix] * vy;
-            float dl = 0.f;
-            if (iy == g.ny - 1 && vy > 0.f) {
-                ex += (float)lF[2 * g.ny + g.nx + ix] * vy;
-                dl = dcoef * vx * vy;
-            }
-            const float wxy = sA[jx] * sA[jy];
-            float *rr = &r.x;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) rr[i] += (ex + dl) * wxy * sA[jz0 + i];
-            dst[o] = r;
-        }
-    }
-}
-
-// The per-sample products of the forward gather live in the last adjoint
-// slab when they fit (that slab is first used after them).
-__host__ __device__ inline bool adj4_gw_in_slab(int nvt, int nt) { return nt <= nvt; }
-
-// Shared-memory bytes of k_adj_cell4: those of k_cell4 plus two slabs, the
-// saved correction sums and one per-jx table.
-__host__ __device__ inline size_t adj4_smem_bytes(int nv, int nvt, int nt)
-{
-    size_t off = (cell4_smem_bytes(nv, nvt, adj4_gw_in_slab(nvt, nt) ? 0 : nt) + 15) & ~(size_t)15;
-    return off + 2 * sizeof(float) * nvt + sizeof(float) * (16 + nv);
-}
-
-// Forward recompute and adjoint of the per-cell relaxation of one step for
-// every cell (FP32 fast path): lt = dJ/dh~ from lam = dJ/dh^{n+1}.
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1024 / MAXT)
-k_adj_cell4(Geo g, Map4 m, const float *__restrict__ hin, const float *__restrict__ ghost,
-            const ushort4 *__restrict__ pidx, const PlanA<float, uint16_t> *__restrict__ pa,
-            const uint32_t *__restrict__ ent, const int *__restrict__ meta,
-            const uint4 *__restrict__ lrec, const int *__restrict__ lmeta,
-            const float *__restrict__ lam, float *__restrict__ lt,
-            unsigned long long *__restrict__ stats)
-{
-    extern __shared__ __align__(16) char smem_raw[];
-    Cell4Smem S = carve4(smem_raw, g.nv, g.nvt);
-    Adj4 X;
-    {
-        const bool gin = adj4_gw_in_slab(g.nvt, g.nt);
-        size_t off = (cell4_smem_bytes(g.nv, g.nvt, gin ? 0 : g.nt) + 15) & ~(size_t)15;
-        X.B = reinterpret_cast<float4 *>(smem_raw + off);
-        X.C = X.B + g.nvt / 4;
-        X.P = reinterpret_cast<float *>(X.C + g.nvt / 4);
-        X.cxi = X.P + 16;
-        X.lam = lam;
-        X.lt = lt;
-        X.pidx = pidx;
-        X.lrec = lrec;
-        X.lmeta = lmeta;
-        if (gin) S.gw = reinterpret_cast<float *>(X.C);
-    }
-    cell4_setup(g, S);
-    int fallback = 0;
-    for (int kc = blockIdx.x; kc < g.nr; kc += gridDim.x)
-        cell4_cell<true, true>(g, m, cell_of(g, kc), hin, ghost, pa, ent, meta, nullptr, nullptr,
-                               S, fallback, nullptr, 0, &X);
     if (fallback && stats) atomicAdd(stats + 3, (unsigned long long)fallback);
 }
 

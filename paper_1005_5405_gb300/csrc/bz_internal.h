@@ -63,7 +63,7 @@ struct bz_adj_scratch {
     void *pidx16, *pa16;
     int *sc_count, *sc_cursor, *sc_meta;   // counts and cursors of both lists, 2 x nvt;
     uint32_t *sc_ent;                      // headers: forward list, then the loss list
-    uint4 *lrec;         // the loss-term records of the transposed update
+    uint2 *lrec;         // the loss-term records of the transposed update
     int map[3];          // Q, K, J
     // The fast path's plan runs on a side stream beside the forward walls.
     cudaStream_t side;
@@ -75,7 +75,7 @@ struct bz_adj_scratch {
     void *pidx16b, *pa16b;
     int *sc_countb, *sc_cursorb, *sc_metab;
     uint32_t *sc_entb;
-    uint4 *lrecb;
+    uint2 *lrecb;
     int64_t *step2;
     int64_t pre_step, last_step;
     cudaEvent_t cell_done;
