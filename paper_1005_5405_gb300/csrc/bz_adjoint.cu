@@ -88,8 +88,8 @@ bz_status setup_generic(bz_adj_scratch *a, const bzk::Geo &g, int nsm, int optin
 }
 
 // The FP32 quad kernel applies when the forward fast path's conditions hold
-// (velocity axis a multiple of 4, 16-bit node indices, 15-bit sample
-// indices) and the two extra slabs fit in shared memory.
+// (velocity axis a multiple of 4, 15-bit sample indices) and three slabs fit in
+// shared memory (which keeps node indices below 14 bits: byte offsets of 16).
 bz_status prepare_fast(bz_adj_scratch *a, const bzk::Geo &g, int nsm, int optin)
 {
     const int N = g.nv, Q = N * N / 4;
