@@ -753,7 +753,10 @@ bz_status configure_relax(bz_handle *H)
     // one, and more CTAs per SM instead.
     const int nseg = sizeof(R) == 8 ? 1 : std::min(std::max(1, 512 / N2), std::min(N, 8));
     H->rx_nseg = nseg;
-    H->rx_T = (N2 * nseg + 31) / 32 * 32;
+    int dev = 0, smem_sm = 0;
+    BZ_CUDA(cudaGetDevice(&dev));
+    BZ_CUDA(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    H->rx_T = H->per_cell ? (N2 * nseg + 31) / 32 * 32 : bzk::rx_threads<R>(N, g.nvt, nseg, g.nt, (size_t)smem_sm);
     H->rx_smem = bzk::rx_smem<R>(nullptr, nullptr, N, g.nvt, H->rx_T, H->per_cell ? 0 : g.nt);
     if (H->rx_smem > (size_t)H->smem_optin) return BZ_OK;
     H->rx_minb = 1;

@@ -93,7 +93,7 @@ bz_status scratch_address(int dev, unsigned char **out)
 // products fit a block's shared memory and the destination-sorted terms fit
 // the scratch array (up to about 36000 FP64 or 48000 FP32 samples): no
 // shared-memory atomics.  64^2 x 24^3 FP32, 10^4 samples: 1052
-// -> 769 us a call.
+// -> 630 us a call.
 // Returns false (nothing launched) otherwise; *e is the launches' status.
 template <typename R>
 bool run_relax(const bzk::Geo &g, unsigned char *scr, const int64_t *stepp, int64_t step, const void *hin, void *hout,
@@ -103,7 +103,10 @@ bool run_relax(const bzk::Geo &g, unsigned char *scr, const int64_t *stepp, int6
     const int N2 = g.nv * g.nv;
     if (g.nv > bzk::kRxMaxN || N2 > (f64 ? 512 : 1024)) return false;
     const int nseg = f64 ? 1 : std::min(std::max(1, 512 / N2), std::min(g.nv, 8));
-    const int T = (N2 * nseg + 31) / 32 * 32;
+    int dev = 0, smem_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const int T = bzk::rx_threads<R>(g.nv, g.nvt, nseg, g.nt, (size_t)smem_sm);
     const size_t smem = bzk::rx_smem<R>(nullptr, nullptr, g.nv, g.nvt, T, g.nt);
     if (smem > (size_t)optin) return false;
     bzk::RxPlans<R> A{};
