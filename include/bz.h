@@ -122,7 +122,8 @@ typedef struct {
     double dt, dx, dy, dv, eps, kcoll;
     int64_t nodes;          /* nx*ny*nv^3 */
     int64_t state_bytes;    /* one state buffer */
-    int64_t step;           /* steps taken so far (time t = step * dt) */
+    int64_t step;           /* steps taken so far (time t = step * dt); after steps captured
+                               by the caller, as of the last bz_get_state or bz_stats */
     int32_t nr, nvt;        /* cells, velocity nodes */
     int32_t dtype;
     int32_t threads_per_cell, smem_bytes;  /* per-cell kernel launch shape */
@@ -154,7 +155,13 @@ bz_status bz_destroy(bz_handle *h);
  * reduces the moments.  On the FP32 active-node path the sample sets of
  * bz_info.plan_batch steps are built ahead in one batch (they depend on the
  * step number only), so the step that starts a batch carries its cost.
- * Asynchronous on `stream`. */
+ * Asynchronous on `stream`.
+ * Steps may be captured into a caller's CUDA graph: an even number of them, so
+ * that a replay finds its input in the buffer where the last one left it.  A
+ * replay takes the steps that follow the device's step counter, whatever steps
+ * were captured; replays may alternate with calls that take an even number of
+ * steps in all.  After a capture each step of the handle builds its own plan, and
+ * bz_get_state waits for `stream` to report the step. */
 bz_status bz_step(bz_handle *h, int32_t nsteps, void *stream);
 
 /* Like bz_step with the sub-steps chosen by `flags` (BZ_DO_STREAM,

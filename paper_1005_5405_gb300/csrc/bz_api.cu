@@ -152,7 +152,14 @@ struct bz_handle {
     // The cells with separate increments (bz_relax.cuh): FP64 states, odd axes
     // and per-cell sets; its plans cover steps [rx_lo, rx_hi).
     bool relax = false;
-    bool captured = false;              // the caller is capturing the stream: no plans built ahead
+    // The caller has captured steps of this handle (replays: sticky).  Their
+    // replays move the device's step counter and the buffers' corrections
+    // without the host, so from then on each step's plan is built from the
+    // device counter in the step itself, both buffers count as carrying
+    // corrections (mu is zero where they do not), and moments are taken anew.
+    // step_plans: the step being enqueued builds its own plan; graph_plans:
+    // so do the two-step graphs.
+    bool replays = false, step_plans = false, graph_plans = false;
     int rx_T = 0, rx_nseg = 1, rx_grid = 0, rx_K = 0, rx_minb = 1;
     size_t rx_smem = 0;
     void *rx_pa = nullptr;
@@ -348,11 +355,14 @@ bz_status configure_cell4(bz_handle *H)
 // Active-node path with deferred correction (bz_lazy.cuh)
 // ---------------------------------------------------------------------
 
+// Whether buffer x may carry pending corrections.
+bool pending(const bz_handle *H, int x) { return H->lazy_buf[x] || (H->replays && H->lazy); }
+
 // A buffer's pending corrections are applied in place (paths that read
 // corrected states call this first).
 bz_status materialize_if_lazy(bz_handle *H, int x, cudaStream_t s)
 {
-    if (!H->lazy_buf[x]) return BZ_OK;
+    if (!pending(H, x)) return BZ_OK;
     const Geo &g = H->g;
     bzk::k_lz_materialize<<<std::min(g.nr, H->nsm * 8), 256, 0, s>>>(
         g, nullptr, (const float *)H->h[x], H->mu[x], (float *)H->h[x], nullptr);
@@ -388,7 +398,7 @@ bool copy_corrected(bz_handle *H, int x, void *dst, cudaStream_t s)
 // Buffer x is about to be overwritten by a path that writes corrected states.
 bz_status drop_lazy(bz_handle *H, int x, cudaStream_t s)
 {
-    if (!H->lazy_buf[x]) return BZ_OK;
+    if (!pending(H, x)) return BZ_OK;
     BZ_CUDA(cudaMemsetAsync(H->mu[x], 0, sizeof(float) * 8 * (size_t)H->g.nr, s));
     H->lazy_buf[x] = false;
     return BZ_OK;
@@ -1043,7 +1053,7 @@ bz_status launch_step(bz_handle *H, cudaStream_t s, bool fused, bool do_stream, 
     using V4 = typename bzk::Idx4<I>::type;
     using PA = bzk::PlanA<R, I>;
     if constexpr (sizeof(R) == 4) {
-        const bool ahead = H->ahead_K > 0 && !H->captured;
+        const bool ahead = H->ahead_K > 0 && !H->step_plans;
         if (fused && H->lazy) return launch_lazy(H, s, true, false, ahead);
         // The relaxation alone on the active-node kernel (no streaming).
         if (!fused && do_collide && !do_stream && H->lazy) return launch_lazy(H, s, true, true, ahead);
@@ -1059,7 +1069,7 @@ bz_status launch_step(bz_handle *H, cudaStream_t s, bool fused, bool do_stream, 
         bzk::k_walls<R><<<g.nfaces, bzk::kWallThreads, 0, s>>>(g, H->d_step, hin, (R *)H->ghost, H->nw, nullptr);
         BZ_LAUNCHED(H);
     }
-    const bool relax = H->relax && (H->per_cell || !H->captured);
+    const bool relax = H->relax && (H->per_cell || !H->step_plans);
     if (fused && relax) return launch_relax<R>(H, s, true, hin, hout);
     if ((do_collide || fused) && !H->per_cell && !relax) {
         ProfScope ps(H, 1, s);
@@ -1532,6 +1542,25 @@ bz_status one_step(bz_handle *H, cudaStream_t s, bool fused, bool ds, bool dc)
                     : launch_step<float, int>(H, s, fused, ds, dc);
 }
 
+bool is_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+// The step counter of a handle whose steps were captured by a caller, read
+// from the device (after the work on s).
+bz_status read_step(bz_handle *H, cudaStream_t s)
+{
+    if (!H->replays || is_capturing(s)) return BZ_OK;
+    int64_t n = 0;
+    BZ_CUDA(cudaMemcpyAsync(&n, H->d_step, sizeof(n), cudaMemcpyDeviceToHost, s));
+    BZ_CUDA(cudaStreamSynchronize(s));
+    H->step = n;
+    return BZ_OK;
+}
+
 bool graphs_enabled()
 {
     const char *e = getenv("BZ_GRAPH");
@@ -1649,16 +1678,21 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     // A graph that the caller captures may be replayed at any step: it holds
     // the kernels that build each step's plan from the device step counter,
-    // not a batch of plans for the steps of the capture.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-    H->captured = cap != cudaStreamCaptureStatusNone;
+    // not a batch of plans for the steps of the capture; and so do the steps
+    // after it, as the host no longer knows the counter.
+    const bool capturing = is_capturing(s);
+    if (capturing) H->replays = true;
+    H->step_plans = H->replays;
+    if (H->replays && !capturing && !H->graph_plans) {
+        drop_graphs(H);                  // (those hold copies of plans built ahead)
+        H->graph_plans = true;
+    }
     bool fused = flags == 0;
     bool ds = (flags & BZ_DO_STREAM) || (flags & BZ_SPLIT);
     bool dc = (flags & BZ_DO_COLLIDE) || (flags & BZ_SPLIT);
     if (ds && dc && !H->ht) BZ_TRY(dalloc(&H->ht, H->esz * (size_t)H->g.nr * H->g.nvt));
     int32_t n = 0;
-    if (fused && nsteps >= 2 && graphs_enabled() && !H->captured) {
+    if (fused && nsteps >= 2 && graphs_enabled() && !capturing) {
         // The captured steps read the buffers as they are now: bring the
         // pair into the state the steps leave it in before capturing.
         if (!H->lazy) {
@@ -1667,7 +1701,7 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
         }
         if (!H->graph[H->cur]) BZ_TRY(capture_pair(H));
         for (; n + 1 < nsteps; n += 2) {
-            BZ_TRY(ensure_plans(H, s, H->step, 2));
+            if (!H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 2));
             if (H->prof) BZ_TRY(arm_profiled_graph(H, H->cur));
             BZ_CUDA(cudaGraphLaunch(H->graph[H->cur], s));
             H->step += 2;
@@ -1679,7 +1713,7 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
     // The steps that run the active-node kernel or the cells with separate increments.
     const bool planned = fused || (dc && (!ds || H->relax));
     for (; n < nsteps; ++n) {
-        if (planned && !H->captured) BZ_TRY(ensure_plans(H, s, H->step, 1));
+        if (planned && !H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 1));
         BZ_TRY(one_step(H, s, fused, ds, dc));
     }
     return BZ_OK;
@@ -1695,13 +1729,13 @@ bz_status bz_moments(bz_handle *H, double *out, void *stream)
     if (!H || !out) return fail(BZ_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
     const Geo &g = H->g;
-    if (!H->mom_valid) {
+    if (!H->mom_valid || H->replays) {
         int grid = std::min(g.nr, H->nsm * 8);
         if (H->dtype == BZ_F64)
             bzk::k_moments<double><<<grid, bzk::kMomThreads, 0, s>>>(g, (const double *)H->h[H->cur], H->mom);
         else
             bzk::k_moments<float><<<grid, bzk::kMomThreads, 0, s>>>(g, (const float *)H->h[H->cur], H->mom,
-                                                                   H->lazy_buf[H->cur] ? H->mu[H->cur] : nullptr);
+                                                                   pending(H, H->cur) ? H->mu[H->cur] : nullptr);
         BZ_LAUNCHED(H);
         H->mom_valid = true;
     }
@@ -1743,14 +1777,17 @@ bz_status bz_lid_shear(bz_handle *H, double *out, void *stream)
 bz_status bz_get_state(bz_handle *H, void *dst, int64_t *step, void *stream)
 {
     if (!H || !dst) return fail(BZ_EINVAL, "NULL argument");
-    if (H->lazy_buf[H->cur] && copy_corrected(H, H->cur, dst, (cudaStream_t)stream)) {
+    if (pending(H, H->cur) && copy_corrected(H, H->cur, dst, (cudaStream_t)stream)) {
         BZ_CUDA(cudaGetLastError());
     } else {
         BZ_TRY(materialize_if_lazy(H, H->cur, (cudaStream_t)stream));
         BZ_CUDA(cudaMemcpyAsync(dst, H->h[H->cur], H->esz * (size_t)H->g.nr * H->g.nvt,
                                 cudaMemcpyDefault, (cudaStream_t)stream));
     }
-    if (step) *step = H->step;
+    if (step) {
+        BZ_TRY(read_step(H, (cudaStream_t)stream));
+        *step = H->step;
+    }
     return BZ_OK;
 }
 
@@ -1823,6 +1860,7 @@ bz_status bz_stats(bz_handle *H, int64_t out[8])
     unsigned long long d[9];
     BZ_CUDA(cudaDeviceSynchronize());
     BZ_CUDA(cudaMemcpy(d, H->stats, sizeof(d), cudaMemcpyDeviceToHost));
+    BZ_TRY(read_step(H, nullptr));
     for (int i = 0; i < 8; ++i) out[i] = (int64_t)d[i];
     out[0] = H->step;
     out[4] = H->launches;
