@@ -923,15 +923,67 @@ __device__ __forceinline__ void lz_solve_fallback(const Geo &g, const float (&P)
     for (int k = 0; k < 5; ++k) mu[k] = m[k];
 }
 
+// Moments of h^{n+1} (Eqs. densita..sforzi) of an FP32 cell from the sums X of N_c
+// over the 30 monomials, the rounding errors Xl of the first ten, the
+// equilibrium sums e0 and the correction mu: sum w h phi = sum N_c phi + sum_a
+// mu_a (E0 + eps sum N_c psi_a phi).  One warp: lane b sums moment b and writes
+// output b.  Every value that ends in an output is a float and its rounding error.
+// (With every operation rounded to FP32 the moments after one step were 1.08e-7 off
+// at 15 nodes per axis and 7.7e-8 at 30, where FP32 sums over the stored result,
+// k_cell's, are 9.1e-8 and 6.0e-8 off; now 8.4e-8 and 4.6e-8, at the same time
+// per step.  In FP64 the chain of about 25 operations took 5 % of a step of 192^2 x 18^3.)
+__device__ __forceinline__ void lz_moments(const float *X, const float *Xl, const float *e0,
+                                           const unsigned char *px, const float (&mu)[5], float eps,
+                                           double *__restrict__ mom)
+{
+    const unsigned all = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    float m = 0.f, ml = 0.f;                           // moment b: m + ml
+    if (lane < 10) {
+        float d = Xl[lane];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const int x = px[k * 16 + lane];
+            d = fmaf(mu[k], fmaf(eps, X[x], e0[x]), d);
+        }
+        two_sum(X[lane], d, m, ml);
+    }
+    const float rho = __shfl_sync(all, m, 0), rl = __shfl_sync(all, ml, 0);
+    const float n = fmaf(eps, rho, 1.f), nl = fmaf(eps, rl, fmaf(eps, rho, 1.f - n)), in = 1.f / n;
+    // (2/3) tr - rho, tr = sum of the second moments
+    float tr, t1, t2, e1, b, bl;
+    two_sum(__shfl_sync(all, m, 4), __shfl_sync(all, m, 5), t1, e1);
+    two_sum(t1, __shfl_sync(all, m, 6), tr, t2);
+    const float trl = (e1 + t2) + ((__shfl_sync(all, ml, 4) + __shfl_sync(all, ml, 5)) + __shfl_sync(all, ml, 6));
+    constexpr float c = 2.f / 3.f, cl = (float)(2.0 / 3.0 - (double)c);
+    const float p = c * tr, pl = fmaf(c, tr, -p) + fmaf(c, trl, cl * tr);
+    two_sum(p, -rho, b, bl);
+    bl += pl - rl;
+    // over n: lanes 1-3 their moment, lane 4 the above
+    const float h = lane == 4 ? b : m, hl = lane == 4 ? bl : ml;
+    const float q = h * in, ql = (fmaf(-q, n, h) + fmaf(-q, nl, hl)) * in;
+    const float u0 = __shfl_sync(all, q, 1), u1 = __shfl_sync(all, q, 2), u2 = __shfl_sync(all, q, 3);
+    const float mq = __shfl_sync(all, m, lane - 1 & 31), mql = __shfl_sync(all, ml, lane - 1 & 31);
+    const float ua = lane == 5 || lane == 8 || lane == 9 ? u0 : lane == 6 || lane == 10 ? u1 : u2;
+    const float ub = lane == 5 ? u0 : lane == 6 || lane == 8 ? u1 : u2;
+    float o = 2.f * mq, ol = fmaf(-2.f * eps * n * ua, ub, 2.f * mql);
+    if (lane < 5) {
+        o = lane == 0 ? m : q;
+        ol = lane == 0 ? ml : ql;
+    }
+    if (lane == 4) ol -= c * eps * (u0 * u0 + u1 * u1 + u2 * u2);
+    if (lane < 11) mom[lane] = (double)o + (double)ol;
+}
+
 // Correction and output moments of one cell from the 26 sums T (of the
-// post-collision N_c = N + dN; the row has room for the 30-entry vector X)
-// and D (of the collision increment dN), both in shared memory: mu to
-// mu_out, moments to mom.  Called by all 32 lanes of a warp: every lane solves
-// the 5 x 5 system (the lanes share its residual), then lane b sums moment b
-// and writes output b.  (With the moments summed by one lane, through arrays
+// post-collision N_c = N + dN; the row has room for the 30-entry vector X), their
+// rounding errors Tl and D (of the collision increment dN), all in shared memory:
+// mu to mu_out, moments to mom.  Called by all 32 lanes of a warp: every lane
+// solves the 5 x 5 system (the lanes share its residual), then lane b sums moment
+// b and writes output b.  (With the moments summed by one lane, through arrays
 // in local memory, a solve took 5-8 thousand cycles.)
-__device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, float *T, const float *D,
-                                          const float *e0, const unsigned char (*px)[16], int *fallback)
+__device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, float *T, const float *Tl,
+                                          const float *D, const float *e0, const unsigned char *px, int *fallback)
 {
     const int lane = threadIdx.x & 31;
     if (lane >= kLzMono && lane < kLzX) {
@@ -966,32 +1018,7 @@ __device__ __forceinline__ void lz_finish(const Geo &g, const LzArgs &a, int c, 
         a.mu_out[(int64_t)c * 8 + lane] = m;
     }
     if (!a.mom) return;
-    // Moments of h^{n+1}: sum w h phi = sum N_c phi + sum_a mu_a (E0 + eps sum N_c psi_a phi).
-    const float eps = g.epsf;
-    float m = 0.f;
-    if (lane < 10) {
-        m = T[lane];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            const int x = px[k][lane];
-            m += mu[k] * (e0[x] + eps * T[x]);
-        }
-    }
-    // Eqs. densita..sforzi (finalize_moments), output `lane` by lane `lane`.
-    const unsigned all = 0xFFFFFFFFu;
-    const float rho = __shfl_sync(all, m, 0), n = 1.f + eps * rho;
-    const float u0 = __shfl_sync(all, m, 1) / n, u1 = __shfl_sync(all, m, 2) / n, u2 = __shfl_sync(all, m, 3) / n;
-    const float tr = __shfl_sync(all, m, 4) + __shfl_sync(all, m, 5) + __shfl_sync(all, m, 6);
-    const float mq = __shfl_sync(all, m, lane - 1 & 31);
-    const float ua = lane == 5 || lane == 8 || lane == 9 ? u0 : lane == 6 || lane == 10 ? u1 : u2;
-    const float ub = lane == 5 ? u0 : lane == 6 || lane == 8 ? u1 : u2;
-    float o = 2.f * mq - 2.f * eps * n * ua * ub;
-    if (lane == 0) o = rho;
-    if (lane == 1) o = u0;
-    if (lane == 2) o = u1;
-    if (lane == 3) o = u2;
-    if (lane == 4) o = ((2.f / 3.f) * tr - rho) / n - (2.f * eps / 3.f) * (u0 * u0 + u1 * u1 + u2 * u2);
-    if (lane < 11) a.mom[(int64_t)c * 11 + lane] = (double)o;
+    lz_moments(T, Tl, e0, px, mu, g.epsf, a.mom + (int64_t)c * 11);
 }
 
 // The (v_y, v_z) part of a cell's pending correction at a thread's nodes (jy;
@@ -1523,13 +1550,16 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                 two_sum(d, H.dpart[db][k][w][lane], d, e);
                 dc = __fadd_rn(dc, e);
             }
-            float tt, te;
+            float tt, te, hi, lo;
             two_sum(f, d, tt, te);
-            H.ftot[fb][k][0][lane] = __fadd_rn(tt, __fadd_rn(te, __fadd_rn(fc, dc)));
+            two_sum(tt, __fadd_rn(te, __fadd_rn(fc, dc)), hi, lo);
+            H.ftot[fb][k][0][lane] = hi;
+            H.ftot[fb][k][1][lane] = lo;
             H.dpart[db][k][0][lane] = __fadd_rn(d, dc);
         }
         __syncwarp();
-        lz_finish(g, a, cell_of(g, kc), H.ftot[fb][k][0], H.dpart[db][k][0], H.e0, H.px, &fallback);
+        lz_finish(g, a, cell_of(g, kc), H.ftot[fb][k][0], H.ftot[fb][k][1], H.dpart[db][k][0], H.e0, &H.px[0][0],
+                  &fallback);
         __syncwarp();
         // The slots take the increment sums of a later group (atomically).
         for (int i = lane; i < kLzDParts * 32; i += 32) (&H.dpart[db][k][0][0])[i] = 0.f;

@@ -38,6 +38,7 @@ struct RxSmem {
     R *e0;                  // [32]: equilibrium sums of the 30 monomials
     R *part;                // [warps][32] partial sums; redraw queue of the per-cell sampler
     R *X, *D;               // [32] totals of N_c over the 30 monomials, [8] of dN
+    R *Xl;                  // [32] rounding errors of X (FP32)
     R *mu;                  // [8]
     R *h, *d, *gw;          // slabs of h~ and dN; products of the shared set
     unsigned char *px;      // [5][16] lz_psiphi
@@ -63,6 +64,7 @@ __host__ __device__ inline size_t rx_smem(RxSmem<R> *s, char *base, int N, int n
     x.part = take((size_t)(T / 32) * 32);
     x.X = take(32);
     x.D = take(8);
+    x.Xl = take(sizeof(R) == 4 ? 32 : 0);
     x.mu = take(8);
     x.px = (unsigned char *)(base + off);
     off += 80;
@@ -216,6 +218,10 @@ __device__ __forceinline__ void rx_finish(const Geo &g, const RxSmem<R> &S, doub
         S.mu[lane] = m;
     }
     if (!mom) return;
+    if constexpr (sizeof(R) == 4) {
+        lz_moments(X, S.Xl, S.e0, S.px, mu, g.epsf, mom);
+        return;
+    }
     const R eps = (R)g.eps;
     R m = R(0);
     if (lane < 10) {
@@ -639,7 +645,9 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
                     two_sum(f, S.part[w * 32 + lane], f, e);
                     fc = __fadd_rn(fc, e);
                 }
-                tot = __fadd_rn(f, fc);
+                float lo;
+                two_sum(f, fc, tot, lo);
+                S.Xl[lane] = lo;
             } else {
                 for (int w = 0; w < cwarps; ++w) tot += S.part[w * 32 + lane];
             }
