@@ -213,15 +213,16 @@ __device__ __forceinline__ SampleOut draw_sample(const Geo &g, int64_t step, uin
 
 // The same sample in FP32, for FP32 states on uniform velocity grids.  The
 // coordinates that pick nodes are computed in FP32 with a bounded error: the
-// uniforms and k_z are rounded once from their integers, -ln u takes the
-// rounding of u to first order, sin(theta) = 2 sqrt(u (1 - u)), and the angles
+// uniforms and k_z are rounded once from their integers, -ln u comes from
+// log1pf of an exact complement, sin(theta) = 2 sqrt(u (1 - u)), and the angles
 // 2 pi u are split into a float part for sincospif and an exact remainder
-// added to first order.  With CUDA's 1-ulp bounds for logf and sincospif this
-// keeps every coordinate of v and v1 within 1.5e-6 of its exact value and
-// every coordinate of v* and v1* within 2.7e-5 (|v| < 4.8 by the Box-Muller
+// added to first order.  With CUDA's 1-ulp bounds for log1pf and sincospif this
+// keeps every coordinate of v and v1 within 1.3e-6 of its exact value and
+// every coordinate of v* and v1* within 2.4e-5 (|v| < 4.8 by the Box-Muller
 // radius at the smallest uniform).  A coordinate closer to a
 // cell face than about four times its bound (kFastMarginA / kFastMarginB, in
-// velocity units, plus the rounding of the cell coordinate itself) sets
+// velocity units, plus the rounding of the cell coordinate itself: two factors and
+// three operations, 2.7e-7 of the n cells of the axis) sets
 // *redo: the caller draws that sample again with draw_sample.  Every other
 // sample selects exactly the nodes of the FP64 computation.  W = cw |s|
 // carries the FP32 error of s (at most 1.6e-5 absolute).
@@ -233,15 +234,21 @@ __device__ __forceinline__ float u01f(uint32_t x)
 {
     return __fmaf_rn((float)(x & 255u) + 0.5f, 0x1p-32f, (float)(x >> 8) * 0x1p-24f);
 }
-// -ln u for u = (x + 1/2) 2^-32: the logarithm of u rounded to float, uf, and
-// to first order the rounding error u - uf (exact; at most 2^-25, so that
-// 1/uf may be 2 - uf: within 2e-8 of the result, which is at least 0.69 where
-// that is off, and exact to 1e-8 of itself as u nears 1).
+// -ln u for u = (x + 1/2) 2^-32, without a branch: u = m 2^-k with m in [1/2, 1), so
+// -ln u = k ln 2 - ln(1 - v) with v = 1 - m, which the integers give exactly
+// and which is rounded once; from u = 1/2 on it is log1p of the exact complement.  (The
+// logarithm of u rounded to float, with its rounding error added to first order, is
+// off by up to 1.2e-7 of the result where that is small, against 0.6e-7 for 1 - u
+// below 2^-8; the two functions with a branch take 7.20 ms for four steps of 64^2 x
+// 24^3 with 10^4 samples per cell, this 6.81.)
 __device__ __forceinline__ float neglog_u01f(uint32_t x)
 {
-    const float hi = (float)(x >> 8) * 0x1p-24f, lo = (float)(x & 255u) + 0.5f;
-    const float uf = __fmaf_rn(lo, 0x1p-32f, hi), du = __fmaf_rn(lo, 0x1p-32f, hi - uf);
-    return -__fmaf_rn(du, 2.f - uf, logf(uf));
+    const int k = __clz((int)x);                              // 32 for x = 0
+    const uint32_t t = __funnelshift_lc(0u, ~x, (uint32_t)k); // v = (t + 2^(k-1)) 2^-32
+    const float half = __int_as_float((126 + k) << 23);       // 2^(k-1)
+    const float v = __fmaf_rn((float)(t & 255u) + half, 0x1p-32f, (float)(t >> 8) * 0x1p-24f);
+    // ln 2 in two parts
+    return __fmaf_rn((float)k, 0.693147182f, __fmaf_rn((float)k, -1.90465421e-9f, -log1pf(-v)));
 }
 // (sin, cos) of 2 pi u for u = (x + 1/2) 2^-32: with x read as a signed
 // integer the angle is pi t, t = (x + 1/2) 2^-31 in [-1, 1), split exactly
@@ -290,7 +297,7 @@ __device__ __forceinline__ SampleOut draw_sample_fast(const Geo &g, int64_t step
     const float st = 2.f * sqrtf(u01f(b.z) * u01f(~b.z));
     const float k[3] = {st * cp, st * sp, kz};
     const float s = (v1[0] - v[0]) * k[0] + (v1[1] - v[1]) * k[1] + (v1[2] - v[2]) * k[2];
-    const float vmax = g.vmaxf, idv = g.idvf, mt = 2.4e-7f * (float)g.nv;
+    const float vmax = g.vmaxf, idv = g.idvf, mt = 3e-7f * (float)g.nv;
     const float ma = kFastMarginA * idv + mt, mb = kFastMarginB * idv + mt;
     const int n = g.nv;
     bool near = false;
