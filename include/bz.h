@@ -141,7 +141,9 @@ typedef struct {
  * (BZ_EINVAL), rejects grids whose velocity slab does not fit one SM's
  * shared memory (BZ_EUNSUPPORTED), allocates two state buffers and the
  * per-step scratch on the current device (BZ_ENOMEM), and sets h = 0, the
- * uniform equilibrium n0, T0 of Sec. 5.1.  *out is NULL on failure. */
+ * uniform equilibrium n0, T0 of Sec. 5.1.  The active-node path also draws the
+ * sample sets of four steps to size its arrays (the call waits for them).  *out is
+ * NULL on failure. */
 bz_status bz_create(const bz_space *space, const bz_vel *vel, const bz_walls *walls,
                     const bz_params *params, bz_handle **out);
 

@@ -136,6 +136,7 @@ struct bz_handle {
     int *lz_flag = nullptr, *lz_cidx = nullptr, *lz_act = nullptr, *lz_wpre = nullptr;
     int *lz_meta = nullptr, *lz_count = nullptr, *lz_cursor = nullptr, *lz_rowend = nullptr;
     int *lz_dest0 = nullptr;
+    void *lz_base = nullptr, *ahead_base = nullptr, *rx_base = nullptr;   // the arrays of each path (Slab)
     uint32_t *lz_mask = nullptr;
     uint2 *lz_rec = nullptr;
     int lz_mcap = 0, lz_G = 0, lz_T = 0, lz_grid = 0, lz_mprobe = 0, lz_stages = 0;
@@ -187,6 +188,32 @@ bz_status dalloc(T **p, size_t bytes)
     }
     return BZ_OK;
 }
+
+// Several device arrays in one allocation, 256-byte aligned, in the order in
+// which they are added (a cudaMalloc takes some 10 us, and a handle with plans
+// built ahead needs some thirty arrays).  With one allocation each, a probe
+// of the active nodes per step with its own read, and the equilibrium sums node
+// by node on the host, creating a handle of 16^2 x 14^3 took 0.99 ms and of 32^2 x
+// 24^3 1.84 ms; now 0.42 and 0.54 ms.
+struct Slab {
+    std::vector<std::pair<void **, size_t>> at;
+    size_t bytes = 0;
+    template <typename T>
+    void add(T **p, size_t n)
+    {
+        at.push_back({(void **)p, bytes});
+        bytes += (n + 255) / 256 * 256;
+    }
+    // *base (freed by the owner) holds them all; the first `zero` bytes are cleared.
+    bz_status alloc(void **base, size_t zero = 0)
+    {
+        const bz_status st = dalloc(base, bytes);
+        if (st != BZ_OK) return st;
+        for (auto &a : at) *a.first = (char *)*base + a.second;
+        if (zero && cudaMemset(*base, 0, zero) != cudaSuccess) return fail(BZ_ECUDA, "memset failed");
+        return BZ_OK;
+    }
+};
 
 #define BZ_TRY(x)                          \
     do {                                   \
@@ -404,44 +431,6 @@ bz_status drop_lazy(bz_handle *H, int x, cudaStream_t s)
     return BZ_OK;
 }
 
-// Value of monomial k of the 30-entry sum vector of bz_lazy.cuh at (x, y, z).
-double lz_monomial(int k, double x, double y, double z)
-{
-    const double v2 = x * x + y * y + z * z;
-    switch (k) {
-    case 0: return 1.0;
-    case 1: return x;
-    case 2: return y;
-    case 3: return z;
-    case 4: return x * x;
-    case 5: return y * y;
-    case 6: return z * z;
-    case 7: return x * y;
-    case 8: return x * z;
-    case 9: return y * z;
-    case 10: return x * x * x;
-    case 11: return y * y * y;
-    case 12: return z * z * z;
-    case 13: return x * x * y;
-    case 14: return x * x * z;
-    case 15: return x * y * y;
-    case 16: return y * y * z;
-    case 17: return x * z * z;
-    case 18: return y * z * z;
-    case 19: return x * y * z;
-    case 20: return x * x * v2;
-    case 21: return y * y * v2;
-    case 22: return z * z * v2;
-    case 23: return x * y * v2;
-    case 24: return x * z * v2;
-    case 25: return y * z * v2;
-    case 26: return v2;
-    case 27: return x * v2;
-    case 28: return y * v2;
-    default: return z * v2;
-    }
-}
-
 // Velocity axes with a kernel specialised on their length (the others run
 // the kernel that reads it at run time); stretched grids (per-cell Courant
 // factors) have their own instances, specialised for 20 nodes per axis (the
@@ -504,7 +493,7 @@ void launch_lz_kernel(bz_handle *H, const bzk::LzArgs &a, cudaStream_t s)
 // only, not on the state) and the compact arrays get a margin above it.  The
 // largest group of cells per CTA (4, else 2) whose shared memory fits is
 // taken.  Needs the per-axis tables on the device.
-bz_status configure_lazy(bz_handle *H)
+bz_status configure_lazy(bz_handle *H, const bz_grid_tables &tb)
 {
     H->lazy = false;
     const Geo &g = H->g;
@@ -516,44 +505,43 @@ bz_status configure_lazy(bz_handle *H)
     const bool pairs = N % 4 == 2 && N >= 14 && H->dtype == BZ_F32 && !H->per_cell && H->idx16 && nt <= 32768;
     if (!(H->fast || pairs) || N > bzk::kLzMaxN) return BZ_OK;
     if (bzk::lz_planes(N, 512) == 0) return BZ_OK;
-    const size_t mub = sizeof(float) * 8 * (size_t)g.nr;
-    BZ_TRY(dalloc(&H->mu[0], mub));
-    BZ_TRY(dalloc(&H->mu[1], mub));
-    BZ_CUDA(cudaMemset(H->mu[0], 0, mub));
-    BZ_CUDA(cudaMemset(H->mu[1], 0, mub));
-    BZ_TRY(dalloc(&H->lz_idx, sizeof(int4) * (size_t)nt));
-    BZ_TRY(dalloc(&H->lz_pa, sizeof(bzk::PlanA<float, int>) * (size_t)nt));
-    BZ_TRY(dalloc(&H->lz_qc, sizeof(ushort4) * (size_t)nt));
-    BZ_TRY(dalloc(&H->lz_flag, sizeof(int) * nvt));
-    BZ_TRY(dalloc(&H->lz_cidx, sizeof(int) * nvt));
-    BZ_TRY(dalloc(&H->lz_act, sizeof(int) * nvt));
-    BZ_TRY(dalloc(&H->lz_mask, sizeof(uint32_t) * ((nvt + 31) / 32)));
-    BZ_TRY(dalloc(&H->lz_wpre, sizeof(int) * ((nvt + 31) / 32)));
-    BZ_TRY(dalloc(&H->lz_meta, sizeof(int) * bzk::kLzMetaSize));
-    BZ_CUDA(cudaMemset(H->lz_flag, 0, sizeof(int) * nvt));
-    BZ_CUDA(cudaMemset(H->lz_meta, 0, sizeof(int) * bzk::kLzMetaSize));
+    const size_t mub = sizeof(float) * 8 * (size_t)g.nr, words = (nvt + 31) / 32;
+    constexpr int kProbes = 4;
+    int *probe = nullptr;
+    Slab sl;
+    sl.add(&H->mu[0], mub);
+    sl.add(&H->mu[1], mub);
+    sl.add(&H->lz_flag, sizeof(int) * nvt);
+    sl.add(&H->lz_count, sizeof(int) * nvt);
+    sl.add(&H->lz_meta, sizeof(int) * bzk::kLzMetaSize);
+    sl.add(&probe, sizeof(int) * kProbes);
+    const size_t zero = sl.bytes;                // (these start from zero)
+    sl.add(&H->lz_idx, sizeof(int4) * (size_t)nt);
+    sl.add(&H->lz_pa, sizeof(bzk::PlanA<float, int>) * (size_t)nt);
+    sl.add(&H->lz_qc, sizeof(ushort4) * (size_t)nt);
+    sl.add(&H->lz_cidx, sizeof(int) * nvt);
+    sl.add(&H->lz_act, sizeof(int) * nvt);
+    sl.add(&H->lz_mask, sizeof(uint32_t) * words);
+    sl.add(&H->lz_wpre, sizeof(int) * words);
+    sl.add(&H->lz_cursor, sizeof(int) * nvt);
+    sl.add(&H->lz_rowend, sizeof(int) * nvt);
+    sl.add(&H->lz_dest0, sizeof(int) * (size_t)bzk::kLzCollT);
+    sl.add(&H->lz_rec, sizeof(uint2) * ((size_t)4 * nt + (size_t)8 * bzk::kLzCollT));
+    BZ_TRY(sl.alloc(&H->lz_base, zero));
 
     // Active nodes of the sample sets of steps 0..3.
-    int64_t *dstep = nullptr;
-    BZ_TRY(dalloc(&dstep, sizeof(int64_t)));
-    Geo gl = g;
-    gl.swz = 0;
-    const int pb = 256, pg = (nt + pb - 1) / pb;
     int mmax = 0;
-    cudaError_t e = cudaSuccess;
-    for (int64_t st = 0; st < 4 && e == cudaSuccess; ++st) {
-        e = cudaMemcpy(dstep, &st, sizeof(int64_t), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) break;
-        bzk::k_plan<float, int><<<pg, pb>>>(gl, dstep, H->lz_idx, H->lz_pa, nullptr, nullptr);
-        bzk::k_lz_mark<<<pg, pb>>>(nt, H->lz_idx, H->lz_flag);
-        bzk::k_lz_scan<<<1, 1024>>>(nvt, nvt, H->lz_flag, H->lz_cidx, H->lz_act, H->lz_mask,
-                                    H->lz_wpre, H->lz_meta);
-        int m = 0;
-        e = cudaMemcpy(&m, H->lz_meta, sizeof(int), cudaMemcpyDeviceToHost);
-        mmax = std::max(mmax, m);
+    {
+        Geo gl = g;
+        gl.swz = 0;
+        int m[kProbes];
+        bzk::k_lz_probe<<<dim3((nt + 63) / 64, kProbes), 64>>>(gl, H->lz_flag);
+        bzk::k_lz_probe_count<<<(nvt + 1023) / 1024, 1024>>>(nvt, H->lz_flag, kProbes, probe);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpy(m, probe, sizeof(m), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return fail(BZ_ECUDA, "active-node probe failed: %s", cudaGetErrorString(e));
+        for (int x : m) mmax = std::max(mmax, x);
     }
-    cudaFree(dstep);
-    if (e != cudaSuccess) return fail(BZ_ECUDA, "active-node probe failed: %s", cudaGetErrorString(e));
     H->lz_mprobe = mmax;
     // The count varies little from step to step (it is a sum of many nearly
     // independent node hits); a step above the capacity runs the fallback.
@@ -620,12 +608,6 @@ bz_status configure_lazy(bz_handle *H)
         if (H->lz_order_tpb > 0)
             BZ_CUDA(bz_allow_max_smem(nb == 8 ? bzk::k_lz_order<8> : bzk::k_lz_order<16>, H->smem_optin));
     }
-    BZ_TRY(dalloc(&H->lz_count, sizeof(int) * (size_t)nvt));
-    BZ_TRY(dalloc(&H->lz_cursor, sizeof(int) * (size_t)nvt));
-    BZ_TRY(dalloc(&H->lz_rowend, sizeof(int) * (size_t)nvt));
-    BZ_TRY(dalloc(&H->lz_dest0, sizeof(int) * (size_t)bzk::kLzCollT));
-    BZ_TRY(dalloc(&H->lz_rec, sizeof(uint2) * ((size_t)4 * nt + (size_t)8 * bzk::kLzCollT)));
-    BZ_CUDA(cudaMemset(H->lz_count, 0, sizeof(int) * (size_t)nvt));
     // Plans of K steps built ahead at a time (BZ_LAZY_AHEAD=K sets the
     // count, 0 builds each step's plan in the step), their term order over
     // whole runs.  The order kernel's one-warp CTAs (T / NB per plan and
@@ -666,37 +648,33 @@ bz_status configure_lazy(bz_handle *H)
         A.osh = H->lz_G == 4 ? 4 : 3;
         A.recn = (int64_t)4 * nt + (int64_t)8 * bzk::kLzCollT;
         const size_t k = (size_t)K;
-        BZ_TRY(dalloc(&A.idx, sizeof(int4) * k * nt));
-        BZ_TRY(dalloc(&A.pa, sizeof(bzk::PlanA<float, int>) * k * nt));
-        BZ_TRY(dalloc(&A.qc, sizeof(ushort4) * k * nt));
-        BZ_TRY(dalloc(&A.flag, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.cidx, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.act, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.mask, sizeof(uint32_t) * k * ((nvt + 31) / 32)));
-        BZ_TRY(dalloc(&A.wpre, sizeof(int) * k * ((nvt + 31) / 32)));
-        BZ_TRY(dalloc(&A.meta, sizeof(int) * k * bzk::kLzMetaSize));
-        BZ_TRY(dalloc(&A.count, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.cursor, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.rowend, sizeof(int) * k * nvt));
-        BZ_TRY(dalloc(&A.dest0, sizeof(int) * k * bzk::kLzCollT));
-        BZ_TRY(dalloc(&A.rec, sizeof(uint2) * k * (size_t)A.recn));
-        BZ_TRY(dalloc(&A.cnt, sizeof(unsigned long long) * 2 * k));
-        BZ_CUDA(cudaMemset(A.flag, 0, sizeof(int) * k * nvt));
-        BZ_CUDA(cudaMemset(A.count, 0, sizeof(int) * k * nvt));
+        Slab as;
+        as.add(&A.flag, sizeof(int) * k * nvt);
+        as.add(&A.count, sizeof(int) * k * nvt);
+        const size_t zeros = as.bytes;
+        as.add(&A.idx, sizeof(int4) * k * nt);
+        as.add(&A.pa, sizeof(bzk::PlanA<float, int>) * k * nt);
+        as.add(&A.qc, sizeof(ushort4) * k * nt);
+        as.add(&A.cidx, sizeof(int) * k * nvt);
+        as.add(&A.act, sizeof(int) * k * nvt);
+        as.add(&A.mask, sizeof(uint32_t) * k * words);
+        as.add(&A.wpre, sizeof(int) * k * words);
+        as.add(&A.meta, sizeof(int) * k * bzk::kLzMetaSize);
+        as.add(&A.cursor, sizeof(int) * k * nvt);
+        as.add(&A.rowend, sizeof(int) * k * nvt);
+        as.add(&A.dest0, sizeof(int) * k * bzk::kLzCollT);
+        as.add(&A.rec, sizeof(uint2) * k * (size_t)A.recn);
+        as.add(&A.cnt, sizeof(unsigned long long) * 2 * k);
+        BZ_TRY(as.alloc(&H->ahead_base, zeros));
         H->ahead_lo = H->ahead_hi = 0;
     }
     // Equilibrium sums of the 30 monomials (the moments of h^{n+1} need them).
-    std::vector<double> axv(N), axA(N);
-    BZ_CUDA(cudaMemcpy(axv.data(), g.axv, sizeof(double) * N, cudaMemcpyDeviceToHost));
-    BZ_CUDA(cudaMemcpy(axA.data(), g.axA, sizeof(double) * N, cudaMemcpyDeviceToHost));
-    for (int k = 0; k < bzk::kLzX; ++k) {
-        double acc = 0.0;
-        for (int jx = 0; jx < N; ++jx)
-            for (int jy = 0; jy < N; ++jy)
-                for (int jz = 0; jz < N; ++jz)
-                    acc += axA[jx] * axA[jy] * axA[jz] * lz_monomial(k, axv[jx], axv[jy], axv[jz]);
-        H->lz_e0[k] = (float)acc;
+    double E[5] = {0, 0, 0, 0, 0};
+    for (int j = 0; j < N; ++j) {
+        double x = tb.axA[j];
+        for (int k = 0; k < 5; ++k, x *= tb.axv[j]) E[k] += x;
     }
+    for (int k = 0; k < bzk::kLzX; ++k) H->lz_e0[k] = (float)bzk::lz_equilibrium(k, E);
     {
         // The plan is a chain of small latency-bound kernels: its blocks go
         // first when the walls' blocks leave room.
@@ -790,13 +768,15 @@ bz_status configure_relax(bz_handle *H)
         const int64_t per = (int64_t)g.nt * (sizeof(bzk::PlanA<R, uint16_t>) + 8 + 16) + (int64_t)g.nvt * 8;
         const int K = H->rx_K = (int)std::max<int64_t>(2, std::min<int64_t>(32, (32 << 20) / per / 2 * 2));
         H->rx_entn = (int64_t)4 * g.nt + H->rx_T;
-        BZ_TRY(dalloc(&H->rx_pa, sizeof(bzk::PlanA<R, uint16_t>) * (size_t)K * g.nt));
-        BZ_TRY(dalloc(&H->rx_idx, sizeof(ushort4) * (size_t)K * g.nt));
-        BZ_TRY(dalloc(&H->rx_count, sizeof(int) * (size_t)K * g.nvt));
-        BZ_TRY(dalloc(&H->rx_cursor, sizeof(int) * (size_t)K * g.nvt));
-        BZ_TRY(dalloc(&H->rx_meta, sizeof(int) * 2 * K));
-        BZ_TRY(dalloc(&H->rx_ent, sizeof(uint32_t) * (size_t)K * H->rx_entn));
-        BZ_TRY(dalloc(&H->rx_cnt, sizeof(unsigned long long) * 2 * K));
+        Slab sl;
+        sl.add(&H->rx_pa, sizeof(bzk::PlanA<R, uint16_t>) * (size_t)K * g.nt);
+        sl.add(&H->rx_idx, sizeof(ushort4) * (size_t)K * g.nt);
+        sl.add(&H->rx_count, sizeof(int) * (size_t)K * g.nvt);
+        sl.add(&H->rx_cursor, sizeof(int) * (size_t)K * g.nvt);
+        sl.add(&H->rx_meta, sizeof(int) * 2 * K);
+        sl.add(&H->rx_ent, sizeof(uint32_t) * (size_t)K * H->rx_entn);
+        sl.add(&H->rx_cnt, sizeof(unsigned long long) * 2 * K);
+        BZ_TRY(sl.alloc(&H->rx_base));
     }
     H->relax = true;
     return BZ_OK;
@@ -1236,18 +1216,8 @@ void release(bz_handle *H)
     void *st[] = {H->axe, H->axd, H->wlid, H->sx, H->sy};
     for (void *p : st)
         if (p) cudaFree(p);
-    void *lz[] = {H->mu[0], H->mu[1], H->lz_idx, H->lz_pa, H->lz_qc, H->lz_flag, H->lz_cidx,
-                  H->lz_act, H->lz_wpre, H->lz_meta, H->lz_count, H->lz_cursor, H->lz_rowend,
-                  H->lz_dest0, H->lz_mask, H->lz_rec};
-    for (void *p : lz)
-        if (p) cudaFree(p);
-    const bzk::AheadPlans &A = H->ahead;
-    void *ah[] = {A.idx, A.pa, A.qc, A.flag, A.cidx, A.act, A.mask, A.wpre, A.meta, A.count, A.cursor,
-                  A.rowend, A.dest0, A.rec, A.cnt};
-    for (void *p : ah)
-        if (p) cudaFree(p);
-    void *rx[] = {H->rx_pa, H->rx_idx, H->rx_count, H->rx_cursor, H->rx_meta, H->rx_ent, H->rx_cnt};
-    for (void *p : rx)
+    void *slabs[] = {H->lz_base, H->ahead_base, H->rx_base};
+    for (void *p : slabs)
         if (p) cudaFree(p);
     bz_adj_release(&H->adj);
 }
@@ -1510,7 +1480,7 @@ bz_status bz_create(const bz_space *space, const bz_vel *vel, const bz_walls *wa
     g.axv = H->axv;
     g.axA = H->axA;
     g.lid_profile = walls->lid_profile ? H->profile : nullptr;
-    st = configure_lazy(H);
+    st = configure_lazy(H, tb);
     if (st != BZ_OK) return bail(st);
     {
         const char *force = getenv("BZ_KERNEL");

@@ -66,6 +66,25 @@ constexpr unsigned long long kLzWaitNs = 1000000000ull;   // an mbarrier wait gi
 // [3] C (terms per thread).
 constexpr int kLzMetaSize = 4;
 
+// The equilibrium sum of entry k of the 30 from the axis sums E_p = sum A v^p (the
+// three axes are alike).
+__host__ __device__ inline double lz_equilibrium(int k, const double (&E)[5])
+{
+    const double z = E[0], e22 = E[2] * E[2] * z, e31 = E[3] * E[1] * z, e112 = E[1] * E[1] * E[2];
+    double x = z * z * z;                                         // 1
+    if (k >= 1 && k <= 3) x = E[1] * z * z;                       // v_i
+    if (k >= 4 && k <= 6) x = E[2] * z * z;                       // v_i^2
+    if (k >= 7 && k <= 9) x = E[1] * E[1] * z;                    // v_i v_j
+    if (k >= 10 && k <= 12) x = E[3] * z * z;                     // v_i^3
+    if (k >= 13 && k <= 18) x = E[2] * E[1] * z;                  // v_i^2 v_j
+    if (k == 19) x = E[1] * E[1] * E[1];                          // v_x v_y v_z
+    if (k >= 20 && k <= 22) x = E[4] * z * z + 2.0 * e22;         // v_i^2 v^2
+    if (k >= 23 && k <= 25) x = 2.0 * e31 + e112;                 // v_i v_j v^2
+    if (k == 26) x = 3.0 * E[2] * z * z;                          // v^2
+    if (k >= 27) x = E[3] * z * z + 2.0 * E[1] * E[2] * z;        // v_i v^2
+    return x;
+}
+
 // Nodes per streaming thread and stage: four consecutive jz (16-byte loads
 // and stores), or two where rows of N nodes are not multiples of 16 bytes
 // (N = 2 mod 4; before, such grids ran the generic per-cell kernel: ten steps of
@@ -106,6 +125,29 @@ static __global__ void k_lz_mark(int nt, const int4 *__restrict__ idx, int *__re
     if (q.y >= 0) flag[q.y] = 1;
     if (q.z >= 0) flag[q.z] = 1;
     if (q.w >= 0) flag[q.w] = 1;
+}
+
+// The nodes that the sample sets of steps 0, 1, ... map to, step blockIdx.y as bit
+// blockIdx.y of flag, and their numbers per step (the flags cleared again): the
+// compact arrays are sized by a few steps, in two launches and one read.
+static __global__ void k_lz_probe(Geo g, int *__restrict__ flag)
+{
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= g.nt) return;
+    const SampleOut o = draw_sample_cell<float>(g, blockIdx.y, 0xFFFFFFFFu, (uint32_t)l);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        if (o.idx[r] >= 0) atomicOr(flag + o.idx[r], 1 << blockIdx.y);
+}
+static __global__ void k_lz_probe_count(int nvt, int *__restrict__ flag, int steps, int *__restrict__ out)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int f = j < nvt ? flag[j] : 0;
+    if (j < nvt) flag[j] = 0;
+    for (int s = 0; s < steps; ++s) {
+        const int n = __syncthreads_count(f >> s & 1);
+        if (threadIdx.x == 0 && n) atomicAdd(out + s, n);
+    }
 }
 
 // Compact numbering of the marked nodes (ascending node order), one CTA of

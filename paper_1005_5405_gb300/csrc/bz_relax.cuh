@@ -427,19 +427,7 @@ k_relax(const __grid_constant__ Geo g, int nseg, const R *__restrict__ hin, cons
         double E[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) E[k] = __shfl_sync(0xFFFFFFFFu, Ek, k);
-        const double z = E[0], e22 = E[2] * E[2] * z, e31 = E[3] * E[1] * z, e112 = E[1] * E[1] * E[2];
-        double x = z * z * z;                                         // 1
-        if (t >= 1 && t <= 3) x = E[1] * z * z;                       // v_i
-        if (t >= 4 && t <= 6) x = E[2] * z * z;                       // v_i^2
-        if (t >= 7 && t <= 9) x = E[1] * E[1] * z;                    // v_i v_j
-        if (t >= 10 && t <= 12) x = E[3] * z * z;                     // v_i^3
-        if (t >= 13 && t <= 18) x = E[2] * E[1] * z;                  // v_i^2 v_j
-        if (t == 19) x = E[1] * E[1] * E[1];                          // v_x v_y v_z
-        if (t >= 20 && t <= 22) x = E[4] * z * z + 2.0 * e22;         // v_i^2 v^2
-        if (t >= 23 && t <= 25) x = 2.0 * e31 + e112;                 // v_i v_j v^2
-        if (t == 26) x = 3.0 * E[2] * z * z;                          // v^2
-        if (t >= 27) x = E[3] * z * z + 2.0 * E[1] * E[2] * z;        // v_i v^2
-        S.e0[t] = (R)x;
+        S.e0[t] = (R)lz_equilibrium(t, E);
     }
     for (int i = t; i < 50; i += T) S.px[i / 10 * 16 + i % 10] = (unsigned char)lz_psiphi(i / 10, i % 10);
     // The thread's column and its range of jx.
