@@ -127,12 +127,15 @@ typedef struct {
     int32_t nr, nvt;        /* cells, velocity nodes */
     int32_t dtype;
     int32_t threads_per_cell, smem_bytes;  /* per-cell kernel launch shape */
-    int32_t kernel_variant;  /* 0: generic per-cell kernel; 1: FP32 4-node-vector kernel;
+    int32_t kernel_variant;  /* 0: the kernels for any type, axis and sample mode (collision
+                                increments in a slab of their own, or in place where two
+                                slabs do not fit); 1: FP32 4-node-vector kernel;
                                 2: FP32 active-node kernel with deferred correction */
-    int32_t plan_batch;      /* active-node kernel: the sample plans of this many
-                                consecutive steps are built together, by the first step
-                                that needs a plan the last batch does not hold; 0: each
-                                step builds its own plan, or another kernel runs */
+    int32_t plan_batch;      /* shared sample sets: the plans of this many consecutive
+                                steps are built together, by the first step that needs
+                                a plan the last batch does not hold; 0: each step
+                                builds its own plan (also after steps captured by the
+                                caller) */
     int64_t plan_end;        /* with plan_batch > 0: the first step the built plans do not
                                 cover (a step from there on builds the next batch) */
 } bz_info;
@@ -154,8 +157,8 @@ bz_status bz_destroy(bz_handle *h);
  * wall densities from h^n (Eq. bcMax), the shared sample set (Sec. 4.2,
  * Algorithm 2), and one fused kernel that streams (Eq. streaming2D),
  * collides (Eq. collision_step), corrects (Eqs. rinorm_a, correzione) and
- * reduces the moments.  On the FP32 active-node path the sample sets of
- * bz_info.plan_batch steps are built ahead in one batch (they depend on the
+ * reduces the moments.  Where bz_info.plan_batch is not 0 the shared sample
+ * sets of that many steps are built ahead in one batch (they depend on the
  * step number only), so the step that starts a batch carries its cost.
  * Asynchronous on `stream`.
  * Steps may be captured into a caller's CUDA graph: an even number of them, so

@@ -1816,11 +1816,13 @@ bz_status bz_get_info(const bz_handle *H, bz_info *o)
     o->nr = g.nr;
     o->nvt = g.nvt;
     o->dtype = H->dtype;
-    o->threads_per_cell = H->lazy ? H->lz_T : H->fast ? H->threads4 : H->threads;
-    o->smem_bytes = (int32_t)(H->lazy ? H->lz_smem : H->fast ? H->smem4 : H->smem_cell);
+    // (After steps captured by the caller the cells of a shared set run k_cell.)
+    const bool relax = H->relax && (H->per_cell || !H->replays);
+    o->threads_per_cell = H->lazy ? H->lz_T : H->fast ? H->threads4 : relax ? H->rx_T : H->threads;
+    o->smem_bytes = (int32_t)(H->lazy ? H->lz_smem : H->fast ? H->smem4 : relax ? H->rx_smem : H->smem_cell);
     o->kernel_variant = H->lazy ? 2 : H->fast ? 1 : 0;
-    o->plan_batch = H->lazy ? H->ahead_K : 0;
-    o->plan_end = H->lazy && H->ahead_K > 0 ? H->ahead_hi : 0;
+    o->plan_batch = H->replays ? 0 : H->lazy ? H->ahead_K : relax && !H->per_cell ? H->rx_K : 0;
+    o->plan_end = o->plan_batch == 0 ? 0 : H->lazy ? H->ahead_hi : H->rx_hi;
     return BZ_OK;
 }
 
