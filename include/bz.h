@@ -133,9 +133,10 @@ typedef struct {
                                 2: FP32 active-node kernel with deferred correction */
     int32_t plan_batch;      /* shared sample sets: the plans of this many consecutive
                                 steps are built together, by the first step that needs
-                                a plan the last batch does not hold; 0: each step
-                                builds its own plan (also after steps captured by the
-                                caller) */
+                                a plan the last batch does not hold (after a jump of
+                                the step counter only those of the call; below the last
+                                batch those that lead up to it); 0: each step builds
+                                its own plan (also after steps captured by the caller) */
     int64_t plan_end;        /* with plan_batch > 0: the first step the built plans do not
                                 cover (a step from there on builds the next batch) */
 } bz_info;

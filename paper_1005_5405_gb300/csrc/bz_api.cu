@@ -782,25 +782,49 @@ bz_status configure_relax(bz_handle *H)
     return BZ_OK;
 }
 
-// The plans of steps [n, n + K) on stream s unless they cover [n, n + cnt)
-// (never while a stream is being captured).
+// The steps [*lo, *hi) whose plans are built next when the slots hold those of
+// [*lo, *hi) and not all of [n, n + cnt); the call takes `left` steps from n
+// on.  A march builds K at a time.  A sweep that comes down in segments (the
+// replays of a reverse pass) builds the K below the window, so that the
+// next segments find theirs (96 steps in segments of four, 32^2 x 15^3: 10.1 -> 8.2
+// ms, where each segment built K).  After a jump only the call's own steps are
+// known to be wanted: one step there 247 -> 165 us.
+void next_plans(int64_t n, int cnt, int64_t left, int K, int64_t *lo, int64_t *hi)
+{
+    int64_t a = n, b = n + K;
+    if (n < *lo && *lo - n <= K) {
+        b = std::max(*lo, n + cnt);
+        a = std::max<int64_t>(0, b - K);
+    } else if (*lo < *hi && (n < *lo || n > *hi)) {
+        b = n + std::min<int64_t>(K, std::max<int64_t>(left, cnt));
+    }
+    *lo = a;
+    *hi = b;
+}
+
+// The plans of the steps from n on (next_plans) on stream s unless they are
+// there for [n, n + cnt) (never while a stream is being captured).
 template <typename R>
-bz_status ensure_rx_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt)
+bz_status ensure_rx_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt, int64_t left)
 {
     if (n >= H->rx_lo && n + cnt <= H->rx_hi) return BZ_OK;
     const bzk::RxPlans<R> A = rx_plans<R>(H);
     const int K = A.K;
+    int64_t lo = H->rx_lo, hi = H->rx_hi;
+    next_plans(n, cnt, left, K, &lo, &hi);
+    const int m = (int)(hi - lo);
+    H->rx_lo = H->rx_hi = 0;
     ProfScope ps(H, 1, s);
     BZ_CUDA(cudaMemsetAsync(A.cnt, 0, sizeof(unsigned long long) * 2 * K, s));
     BZ_CUDA(cudaMemsetAsync(A.count, 0, sizeof(int) * (size_t)K * A.nvt, s));
-    bzk::k_rx_plan<R><<<dim3((A.nt + 63) / 64, K), 64, 0, s>>>(H->g, A, n);
+    bzk::k_rx_plan<R><<<dim3((A.nt + 63) / 64, m), 64, 0, s>>>(H->g, A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_rx_scan<R><<<K, 1024, 0, s>>>(A);
+    bzk::k_rx_scan<R><<<m, 1024, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_rx_fill<R><<<dim3((A.nt + 255) / 256, K), 256, 0, s>>>(A);
+    bzk::k_rx_fill<R><<<dim3((A.nt + 255) / 256, m), 256, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
-    H->rx_lo = n;
-    H->rx_hi = n + K;
+    H->rx_lo = lo;
+    H->rx_hi = hi;
     return BZ_OK;
 }
 
@@ -837,43 +861,47 @@ bz_status launch_relax(bz_handle *H, cudaStream_t s, bool fused, const R *hin, R
 // nostream: the relaxation alone (BZ_DO_COLLIDE), h~ = h; the walls still
 // run so that the ghost values the kernel reads (times a zero Courant
 // number) are those of the state.
-// The plans of steps [n, n + K) built ahead into the handle's K slots on
-// stream s, unless the slots already cover [n, n + cnt).  Never called while
+// The plans of the steps from n on (next_plans) built ahead into the handle's K
+// slots on stream s, unless the slots already cover [n, n + cnt).  Never called while
 // a stream is being captured (the step graphs hold only k_ahead_take).
-bz_status ensure_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt)
+bz_status ensure_plans(bz_handle *H, cudaStream_t s, int64_t n, int cnt, int64_t left)
 {
     if (H->relax && !H->per_cell)
-        return H->dtype == BZ_F64 ? ensure_rx_plans<double>(H, s, n, cnt) : ensure_rx_plans<float>(H, s, n, cnt);
+        return H->dtype == BZ_F64 ? ensure_rx_plans<double>(H, s, n, cnt, left) : ensure_rx_plans<float>(H, s, n, cnt, left);
     if (!H->lazy || H->ahead_K == 0) return BZ_OK;
     if (n >= H->ahead_lo && n + cnt <= H->ahead_hi) return BZ_OK;
     const bzk::AheadPlans &A = H->ahead;
     const int K = H->ahead_K;
+    int64_t lo = H->ahead_lo, hi = H->ahead_hi;
+    next_plans(n, cnt, left, K, &lo, &hi);
+    const int m = (int)(hi - lo);
+    H->ahead_lo = H->ahead_hi = 0;
     Geo gl = H->g;
     gl.swz = 0;
     ProfScope ps(H, 1, s);
     BZ_CUDA(cudaMemsetAsync(A.cnt, 0, sizeof(unsigned long long) * 2 * K, s));
-    bzk::k_ahead_plan<<<dim3((A.nt + 63) / 64, K), 64, 0, s>>>(gl, A, n);
+    bzk::k_ahead_plan<<<dim3((A.nt + 63) / 64, m), 64, 0, s>>>(gl, A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_ahead_scan<<<K, 1024, 0, s>>>(A, n);
+    bzk::k_ahead_scan<<<m, 1024, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_ahead_remap<<<dim3((A.nt + 255) / 256, K), 256, 0, s>>>(A, n);
+    bzk::k_ahead_remap<<<dim3((A.nt + 255) / 256, m), 256, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_ahead_lscan<<<K, 1024, 0, s>>>(A, n);
+    bzk::k_ahead_lscan<<<m, 1024, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
-    bzk::k_ahead_lfill<<<dim3((A.nt + 255) / 256, K), 256, 0, s>>>(A, n);
+    bzk::k_ahead_lfill<<<dim3((A.nt + 255) / 256, m), 256, 0, s>>>(A, lo);
     BZ_LAUNCHED(H);
     if (H->lz_order_tpb > 0) {
-        const int ch = H->ahead_chunk, nch = (H->lz_cmax + ch - 1) / ch, z0 = (int)(n % K);
+        const int ch = H->ahead_chunk, nch = (H->lz_cmax + ch - 1) / ch, z0 = (int)(lo % K);
         if (H->lz_G == 4)
-            bzk::k_lz_order<8><<<dim3(bzk::kLzCollT / 8, nch, K), 32, bzk::lz_order_smem(ch, 8), s>>>(
+            bzk::k_lz_order<8><<<dim3(bzk::kLzCollT / 8, nch, m), 32, bzk::lz_order_smem(ch, 8), s>>>(
                 bzk::kLzCollT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
         else
-            bzk::k_lz_order<16><<<dim3(bzk::kLzCollT / 16, nch, K), 32, bzk::lz_order_smem(ch, 16), s>>>(
+            bzk::k_lz_order<16><<<dim3(bzk::kLzCollT / 16, nch, m), 32, bzk::lz_order_smem(ch, 16), s>>>(
                 bzk::kLzCollT, H->lz_cmax, ch, A.meta, A.rec, K, z0, A.recn);
         BZ_LAUNCHED(H);
     }
-    H->ahead_lo = n;
-    H->ahead_hi = n + K;
+    H->ahead_lo = lo;
+    H->ahead_hi = hi;
     return BZ_OK;
 }
 
@@ -1671,7 +1699,7 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
         }
         if (!H->graph[H->cur]) BZ_TRY(capture_pair(H));
         for (; n + 1 < nsteps; n += 2) {
-            if (!H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 2));
+            if (!H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 2, nsteps - n));
             if (H->prof) BZ_TRY(arm_profiled_graph(H, H->cur));
             BZ_CUDA(cudaGraphLaunch(H->graph[H->cur], s));
             H->step += 2;
@@ -1683,7 +1711,7 @@ bz_status bz_step_ex(bz_handle *H, int32_t nsteps, uint32_t flags, void *stream)
     // The steps that run the active-node kernel or the cells with separate increments.
     const bool planned = fused || (dc && (!ds || H->relax));
     for (; n < nsteps; ++n) {
-        if (planned && !H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 1));
+        if (planned && !H->step_plans) BZ_TRY(ensure_plans(H, s, H->step, 1, nsteps - n));
         BZ_TRY(one_step(H, s, fused, ds, dc));
     }
     return BZ_OK;
@@ -2224,7 +2252,7 @@ bz_status fan_launch(bz_batch *B, cudaStream_t s, bool advance_step)
 // not cover them yet (the instances step together, so they all need a batch
 // at the same steps): each instance's batch on its branch, forked from and
 // joined back to s.  Never called while a stream is being captured.
-bz_status fan_ensure(bz_batch *B, cudaStream_t s)
+bz_status fan_ensure(bz_batch *B, cudaStream_t s, int64_t left)
 {
     bool need = false;
     for (int i = 0; i < B->n && !need; ++i) {
@@ -2235,7 +2263,7 @@ bz_status fan_ensure(bz_batch *B, cudaStream_t s)
     const int nb = B->branches;
     BZ_CUDA(cudaEventRecord(B->ev[0], s));
     for (int k = 0; k < nb; ++k) BZ_CUDA(cudaStreamWaitEvent(B->br[k], B->ev[0], 0));
-    for (int i = 0; i < B->n; ++i) BZ_TRY(ensure_plans(B->inst[i], B->br[B->owner[i]], B->step[i], 1));
+    for (int i = 0; i < B->n; ++i) BZ_TRY(ensure_plans(B->inst[i], B->br[B->owner[i]], B->step[i], 1, left));
     for (int k = 0; k < nb; ++k) {
         BZ_CUDA(cudaEventRecord(B->ev[1 + k], B->br[k]));
         BZ_CUDA(cudaStreamWaitEvent(s, B->ev[1 + k], 0));
@@ -2639,7 +2667,7 @@ bz_status bz_batch_step(bz_batch *B, int32_t nsteps, void *stream)
             if (e != cudaSuccess) return fail(BZ_ECUDA, "batch graph: %s", cudaGetErrorString(e));
         }
         for (int32_t k = 0; k < nsteps; ++k) {
-            if (B->lz_ahead) BZ_TRY(fan_ensure(B, s));
+            if (B->lz_ahead) BZ_TRY(fan_ensure(B, s, nsteps - k));
             if (B->graph2 && graphs_enabled()) BZ_CUDA(cudaGraphLaunch(B->graph2, s));
             else BZ_TRY(lz_batch_launch(B, s, true));
             for (auto &v : B->step) v += 1;
@@ -2657,7 +2685,7 @@ bz_status bz_batch_step(bz_batch *B, int32_t nsteps, void *stream)
     }
     if (B->mode == 1) {
         for (int32_t k = 0; k < nsteps; ++k) {
-            BZ_TRY(fan_ensure(B, s));
+            BZ_TRY(fan_ensure(B, s, nsteps - k));
             if (graphs_enabled()) {
                 cudaGraphExec_t ex = nullptr;
                 BZ_TRY(fan_graph(B, &ex));
@@ -2784,7 +2812,7 @@ bz_status bz_batch_tune(bz_batch *B, int32_t trial_steps, void *stream, int32_t 
                     t = f / trial_steps;
             }
         } else if (k.mode == 2) {
-            if (batch_set_mode(B, 2, s) == BZ_OK && (!B->lz_ahead || fan_ensure(B, s) == BZ_OK) &&
+            if (batch_set_mode(B, 2, s) == BZ_OK && (!B->lz_ahead || fan_ensure(B, s, 1) == BZ_OK) &&
                 lz_batch_launch(B, s, false) == BZ_OK) {
                 cudaEventRecord(e0, s);
                 bool ok = true;
@@ -2802,7 +2830,7 @@ bz_status bz_batch_tune(bz_batch *B, int32_t trial_steps, void *stream, int32_t 
             cudaGraphExec_t ex = nullptr;
             std::vector<long long> l0(B->n);
             for (int i = 0; i < B->n; ++i) l0[i] = B->inst[i]->launches;
-            bool ok = fan_ensure(B, s) == BZ_OK &&
+            bool ok = fan_ensure(B, s, 1) == BZ_OK &&
                       cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
             bz_status st = ok ? fan_launch(B, B->cap, false) : BZ_ECUDA;
             ok = cudaStreamEndCapture(B->cap, &graph) == cudaSuccess && ok && st == BZ_OK;

@@ -139,8 +139,8 @@ bool run_relax(const bzk::Geo &g, unsigned char *scr, const int64_t *stepp, int6
     *e = cudaMemsetAsync(A.cnt, 0, (size_t)((unsigned char *)A.cursor - (unsigned char *)A.cnt), s);
     if (*e != cudaSuccess) return true;
     bzk::k_rx_plan<R><<<(g.nt + 63) / 64, 64, 0, s>>>(g, A, step);
-    bzk::k_rx_scan<R><<<1, 1024, 0, s>>>(A);
-    bzk::k_rx_fill<R><<<(g.nt + 255) / 256, 256, 0, s>>>(A);
+    bzk::k_rx_scan<R><<<1, 1024, 0, s>>>(A, step);
+    bzk::k_rx_fill<R><<<(g.nt + 255) / 256, 256, 0, s>>>(A, step);
     k<<<std::min(g.nr, nsm * occ), T, smem, s>>>(g, nseg, (const R *)hin, nullptr, A, (R *)hout, mom, nullptr, stepp);
     *e = cudaGetLastError();
     return true;

@@ -291,17 +291,19 @@ __global__ void k_rx_plan(Geo g, RxPlans<R> A, int64_t step0)
     }
 }
 template <typename R>
-__global__ void __launch_bounds__(1024) k_rx_scan(RxPlans<R> A)
+__global__ void __launch_bounds__(1024) k_rx_scan(RxPlans<R> A, int64_t step0)
 {
     __shared__ int part[1024];
-    const int64_t v = (int64_t)blockIdx.x * A.nvt;
-    scatter_scan_body(A.nvt, A.T, A.count + v, A.cursor + v, A.meta + 2 * blockIdx.x, part);
+    const int s = (int)((step0 + blockIdx.x) % A.K);
+    const int64_t v = (int64_t)s * A.nvt;
+    scatter_scan_body(A.nvt, A.T, A.count + v, A.cursor + v, A.meta + 2 * s, part);
 }
 template <typename R>
-__global__ void k_rx_fill(RxPlans<R> A)
+__global__ void k_rx_fill(RxPlans<R> A, int64_t step0)
 {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= A.nt) return;
+    const int s = (int)((step0 + blockIdx.y) % A.K);
     const int C = A.meta[2 * s + 1];
     const ushort4 q = A.idx[(int64_t)s * A.nt + l];
     const unsigned short d[4] = {q.x, q.y, q.z, q.w};
