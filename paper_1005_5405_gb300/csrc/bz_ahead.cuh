@@ -43,7 +43,7 @@ __device__ __forceinline__ int ahead_slot(const AheadPlans &A, int64_t step0, in
 // FP32 sampler of the per-cell sets draws them (uniform velocity grids; a
 // sample near a velocity-cell face is drawn again in FP64), so the node
 // indices are those of the FP64 computation and W carries FP32 rounding.
-__global__ void k_ahead_plan(Geo g, AheadPlans A, int64_t step0)
+static __global__ void k_ahead_plan(Geo g, AheadPlans A, int64_t step0)
 {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t step = step0 + blockIdx.y;
@@ -69,7 +69,7 @@ __global__ void k_ahead_plan(Geo g, AheadPlans A, int64_t step0)
 }
 
 // Compact numbering of the marked nodes: one CTA of 1024 threads per step.
-__global__ void __launch_bounds__(1024) k_ahead_scan(AheadPlans A, int64_t step0)
+static __global__ void __launch_bounds__(1024) k_ahead_scan(AheadPlans A, int64_t step0)
 {
     const int s = ahead_slot(A, step0, blockIdx.x);
     const int64_t v = (int64_t)s * A.nvt, w = (int64_t)s * ((A.nvt + 31) / 32);
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(1024) k_ahead_scan(AheadPlans A, int64_t step0
                   A.meta + s * kLzMetaSize, nullptr);
 }
 
-__global__ void k_ahead_remap(AheadPlans A, int64_t step0)
+static __global__ void k_ahead_remap(AheadPlans A, int64_t step0)
 {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= A.nt) return;
@@ -87,7 +87,7 @@ __global__ void k_ahead_remap(AheadPlans A, int64_t step0)
 }
 
 // Sorted order of the collision terms: one CTA of 1024 threads per step.
-__global__ void __launch_bounds__(1024) k_ahead_lscan(AheadPlans A, int64_t step0)
+static __global__ void __launch_bounds__(1024) k_ahead_lscan(AheadPlans A, int64_t step0)
 {
     const int s = ahead_slot(A, step0, blockIdx.x);
     const int64_t v = (int64_t)s * A.nvt;
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(1024) k_ahead_lscan(AheadPlans A, int64_t step
                    A.rec + s * A.recn, A.dest0 + s * kLzCollT);
 }
 
-__global__ void k_ahead_lfill(AheadPlans A, int64_t step0)
+static __global__ void k_ahead_lfill(AheadPlans A, int64_t step0)
 {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= A.nt) return;
@@ -145,7 +145,7 @@ __device__ __forceinline__ void ahead_take(const AheadPlans &A, int64_t step, in
 
 // The plan of the current step (*stepp) of one handle.  Grid-stride over
 // every array.
-__global__ void k_ahead_take(AheadPlans A, const int64_t *__restrict__ stepp, int4 *__restrict__ idx,
+static __global__ void k_ahead_take(AheadPlans A, const int64_t *__restrict__ stepp, int4 *__restrict__ idx,
                              PlanA<float, int> *__restrict__ pa, int *__restrict__ meta,
                              uint32_t *__restrict__ mask, int *__restrict__ wpre, int *__restrict__ act,
                              uint2 *__restrict__ rec, int *__restrict__ dest0,

@@ -10,6 +10,7 @@
 #include "bz_cell4.cuh"
 #include "bz_batch.cuh"
 #include "bz_lazy.cuh"
+#include "bz_lz_kernels.h"
 #include "bz_ahead.cuh"
 #include "bz_relax.cuh"
 
@@ -128,6 +129,7 @@ struct bz_handle {
     double *axe = nullptr, *axd = nullptr, *wlid = nullptr;
     double *sx = nullptr, *sy = nullptr;
     bool lazy = false;
+    bzk::LzKernel lz_kern = nullptr;
     float *mu[2] = {nullptr, nullptr};
     bool lazy_buf[2] = {false, false};
     int4 *lz_idx = nullptr;
@@ -431,60 +433,15 @@ bz_status drop_lazy(bz_handle *H, int x, cudaStream_t s)
     return BZ_OK;
 }
 
-// Velocity axes with a kernel specialised on their length (the others run
-// the kernel that reads it at run time); stretched grids (per-cell Courant
-// factors) have their own instances, specialised for 20 nodes per axis (the
-// paper's stretched cavities) and run-time lengths otherwise.
-int lz_nv_key(const bz_handle *H) { return H->stretched ? (H->g.nv == 20 || H->g.nv == 18 ? -H->g.nv : -1) : H->g.nv; }
-
-// Calls f with the k_lz instance of a handle: G cells per group, the axis
-// length as a constant where it has an instance, stretched cells, the
-// streaming threads, the bulk-copy ring.
-template <int G, int ST, typename F>
-auto with_lz_kernel(const bz_handle *H, F f)
+// The active-node kernel of a handle with groups of G cells and ST streaming
+// threads.
+bzk::LzKernel lz_kernel(const bz_handle *H, int G, int ST)
 {
-    if constexpr (G == 4 && ST == 256) {
-        if (H->lz_tma && lz_nv_key(H) >= 0)
-            return lz_nv_key(H) == 32 ? f(bzk::k_lz<4, 32, false, 256, true>) : f(bzk::k_lz<4, 0, false, 256, true>);
-    }
-    if (H->g.nv % 4 != 0) {
-        if constexpr (G == 4 && ST == 512)
-            if (lz_nv_key(H) == -18) return f(bzk::k_lz<4, 18, true, 512>);
-        return H->stretched ? f(bzk::k_lz<G, 0, true, ST, false, 2>) : f(bzk::k_lz<G, 0, false, ST, false, 2>);
-    }
-    if constexpr (G == 4 && ST == 512) {
-        if (lz_nv_key(H) == 24) return f(bzk::k_lz<4, 24, false, 512>);
-    } else if constexpr (G == 4) {
-        switch (lz_nv_key(H)) {
-        case 32: return f(bzk::k_lz<4, 32, false, ST>);
-        case 28: return f(bzk::k_lz<4, 28, false, ST>);
-        case 20: return f(bzk::k_lz<4, 20, false, ST>);
-        case 16: return f(bzk::k_lz<4, 16, false, ST>);
-        case -20: return f(bzk::k_lz<4, 20, true, ST>);
-        }
-    }
-    return H->stretched ? f(bzk::k_lz<G, 0, true, ST>) : f(bzk::k_lz<G, 0, false, ST>);
-}
-
-bz_status setup_lz_kernel(bz_handle *H, int G, int ST, size_t smem, int *occ)
-{
-    auto set = [&](auto *k) -> bz_status {
-        BZ_CUDA(bz_allow_max_smem(k, H->smem_optin));
-        BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, bzk::lz_threads(ST), smem));
-        return BZ_OK;
-    };
-    if (ST == 512) return G == 4 ? with_lz_kernel<4, 512>(H, set) : with_lz_kernel<2, 512>(H, set);
-    return G == 4 ? with_lz_kernel<4, 256>(H, set) : with_lz_kernel<2, 256>(H, set);
-}
-
-void launch_lz_kernel(bz_handle *H, const bzk::LzArgs &a, cudaStream_t s)
-{
-    auto go = [&](auto *k) { k<<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(H->g, a); };
-    if (H->lz_T == bzk::lz_threads(512)) {
-        if (H->lz_G == 4) with_lz_kernel<4, 512>(H, go);
-        else with_lz_kernel<2, 512>(H, go);
-    } else if (H->lz_G == 4) with_lz_kernel<4, 256>(H, go);
-    else with_lz_kernel<2, 256>(H, go);
+    const int N = H->g.nv;
+    if (G == 4 && ST == 256 && H->lz_tma && !H->stretched) return bzk::lz_kernel_bulk(N);
+    if (G == 4 && ST == bzk::lz_stream_threads(N))
+        return H->stretched ? bzk::lz_kernel_stretched(N) : bzk::lz_kernel_uniform(N);
+    return bzk::lz_kernel_general(G, ST, H->stretched, bzk::lz_vec(N));
 }
 
 // Decide whether the active-node path applies (FP32 fast path, at most 32
@@ -568,8 +525,11 @@ bz_status configure_lazy(bz_handle *H, const bz_grid_tables &tb)
             if (stages < 3) continue;
             const size_t smem = bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end;
             int occ = 0;
-            BZ_TRY(setup_lz_kernel(H, G, ST, smem, &occ));
+            const bzk::LzKernel kern = lz_kernel(H, G, ST);
+            BZ_CUDA(bz_allow_max_smem(kern, H->smem_optin));
+            BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, bzk::lz_threads(ST), smem));
             if (occ < 1) continue;
+            H->lz_kern = kern;
             H->lz_G = G;
             H->lz_T = bzk::lz_threads(ST);
             H->lz_smem = smem;
@@ -1002,7 +962,7 @@ bz_status launch_lazy(bz_handle *H, cudaStream_t s, bool advance_step = true, bo
         // collision warps start the increment sums.
         a.early_tail = 1;
         if (const char *et = getenv("BZ_LAZY_EARLY_TAIL")) a.early_tail = atoi(et) != 0 ? 1 : 0;
-        launch_lz_kernel(H, a, s);
+        H->lz_kern<<<H->lz_grid, H->lz_T, H->lz_smem, s>>>(g, a);
         BZ_LAUNCHED(H);
     }
     {
@@ -2074,7 +2034,7 @@ struct bz_batch {
     int *d_next = nullptr;                  // one claim counter per velocity grid
     int nseg = 0;
     size_t lz_smem = 0;
-    struct LzClass { int nv, ST, seg0, nseg; size_t smem; };
+    struct LzClass { bzk::LzBatchKernel kern; int nv, seg0, nseg; size_t smem; };
     std::vector<LzClass> lz_classes;        // the segments of each velocity grid
     cudaStream_t lz_side = nullptr;         // the sample plans run here, beside the walls
     cudaEvent_t lz_fork = nullptr, lz_join = nullptr;
@@ -2217,14 +2177,6 @@ bz_status batch_correct_in_place(bz_batch *B, int i, cudaStream_t s)
     BZ_CUDA(cudaGetLastError());
     BZ_CUDA(cudaMemsetAsync(h->mu[b], 0, sizeof(float) * 8 * (size_t)h->g.nr, s));
     return BZ_OK;
-}
-
-// Calls f with the batch kernel instance of a velocity-grid class.
-template <typename F>
-auto with_kbl_lz(int nv, int ST, F f)
-{
-    if (ST == 512) return nv == 24 ? f(bzk::kbl_lz<24, 512>) : f(bzk::kbl_lz<0, 512>);
-    return nv == 20 ? f(bzk::kbl_lz<20, 256>) : nv == 16 ? f(bzk::kbl_lz<16, 256>) : f(bzk::kbl_lz<0, 256>);
 }
 
 // One fan-out step: fork to the branches, each instance's active-node step
@@ -2370,9 +2322,7 @@ bz_status lz_batch_launch(bz_batch *B, cudaStream_t s, bool advance)
         int *nx = B->d_next + k;
         const cudaStream_t sk = k == 0 ? s : B->lz_cls_s[k - 1];
         if (k > 0) BZ_CUDA(cudaStreamWaitEvent(sk, B->lz_go, 0));
-        with_kbl_lz(c.nv, c.ST, [&](auto *kern) {
-            kern<<<B->nsm, bzk::lz_threads(c.ST), c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx);
-        });
+        c.kern<<<B->nsm, bzk::lz_threads(bzk::lz_stream_threads(c.nv)), c.smem, sk>>>(B->d_lzinst, sg4, c.nseg, nx);
         if (k > 0) BZ_CUDA(cudaEventRecord(B->lz_cls_done[k - 1], sk));
     }
     for (size_t k = 1; k < nc; ++k) BZ_CUDA(cudaStreamWaitEvent(s, B->lz_cls_done[k - 1], 0));
@@ -2390,12 +2340,13 @@ bz_status lz_batch_launch(bz_batch *B, cudaStream_t s, bool advance)
 }
 
 // Set-up of the persistent active-node mode (lz_ok stays false when an
-// instance does not run the active-node kernel with groups of four cells).
+// instance does not run the active-node kernel with groups of four cells and
+// its length's streaming threads).
 bz_status lz_batch_prepare(bz_batch *B)
 {
     B->lz_ok = false;
     for (bz_handle *h : B->inst)
-        if (!h->lazy || h->lz_G != 4) return BZ_OK;
+        if (!h->lazy || h->lz_G != 4 || h->lz_T != bzk::lz_threads(bzk::lz_stream_threads(h->g.nv))) return BZ_OK;
     const int n = B->n;
     std::vector<bzk::LzInst> li(n);
     size_t smem = 0;
@@ -2456,17 +2407,14 @@ bz_status lz_batch_prepare(bz_batch *B)
     // instance's groups, the instances with the largest velocity grids (the
     // costliest groups) first.
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-        return B->inst[x]->g.nv != B->inst[y]->g.nv ? B->inst[x]->g.nv > B->inst[y]->g.nv
-                                                    : B->inst[x]->lz_T > B->inst[y]->lz_T;
+        return B->inst[x]->g.nv > B->inst[y]->g.nv;
     });
     std::vector<int4> segs;
     B->lz_classes.clear();
     for (int i : order) {
         const int nv = B->inst[i]->g.nv;
-        const int key = nv == 24 || nv == 20 || nv == 16 ? nv : 0;
-        const int ST = B->inst[i]->lz_T - bzk::kLzCollT;
-        if (B->lz_classes.empty() || B->lz_classes.back().nv != key || B->lz_classes.back().ST != ST)
-            B->lz_classes.push_back({key, ST, (int)segs.size(), 0, 0});
+        if (B->lz_classes.empty() || B->lz_classes.back().nv != nv)
+            B->lz_classes.push_back({bzk::lz_batch_kernel(nv), nv, (int)segs.size(), 0, 0});
         auto &c = B->lz_classes.back();
         c.smem = std::max(c.smem, (size_t)B->inst[i]->lz_smem);
         const int ng = (B->inst[i]->g.nr + 3) / 4, R = std::max(1, (ng + 31) / 32);
@@ -2476,11 +2424,9 @@ bz_status lz_batch_prepare(bz_batch *B)
     bz_handle *h0 = B->inst[0];
     for (const auto &c : B->lz_classes) {
         int occ = 0;
-        BZ_TRY(with_kbl_lz(c.nv, c.ST, [&](auto *kern) -> bz_status {
-            BZ_CUDA(bz_allow_max_smem(kern, h0->smem_optin));
-            BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, bzk::lz_threads(c.ST), c.smem));
-            return BZ_OK;
-        }));
+        BZ_CUDA(bz_allow_max_smem(c.kern, h0->smem_optin));
+        BZ_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &occ, c.kern, bzk::lz_threads(bzk::lz_stream_threads(c.nv)), c.smem));
         if (occ < 1) return BZ_OK;
     }
     BZ_CUDA(bz_allow_max_smem(bzk::kbl_fb_cell4, h0->smem_optin));

@@ -105,7 +105,7 @@ __host__ __device__ constexpr int lz_planes(int N, int ST)
 
 // Streaming threads for N nodes per axis: 512 where that raises the busy
 // share by more than 1.4 (above), or where a plane needs them, else 256.
-constexpr int lz_stream_threads(int N)
+__host__ __device__ constexpr int lz_stream_threads(int N)
 {
     const int s2 = lz_planes(N, 256), s5 = lz_planes(N, 512);
     return s2 == 0 || 10 * s5 * 256 > 14 * s2 * 512 ? 512 : 256;
