@@ -331,8 +331,8 @@ bz_status bz_profile_read(bz_handle *h, double ms[4], int64_t launches[4]);
  * For the active-node kernel (variant 2) an item is an iteration of its two
  * roles and the points are: iteration start, streaming done, collision
  * terms done, their sums done, write-back done, correction and moments of
- * the group two back done (the first two from a streaming thread, the next
- * three from a collision thread).  out: at least 72 int64, host; row-major
+ * the group two back done (the first two from a streaming thread, the others
+ * from a collision thread, whose first work of an iteration is the last point).  out: at least 72 int64, host; row-major
  * [item][point].  BZ_ESTATE if not enabled. */
 bz_status bz_phase_clocks(bz_handle *h, int64_t *out, int32_t n);
 

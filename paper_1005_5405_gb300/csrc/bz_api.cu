@@ -521,8 +521,8 @@ bz_status configure_lazy(bz_handle *H, const bz_grid_tables &tb)
             const int VW = bzk::lz_vec(N), S = bzk::lz_planes(N, ST) * (N * N / VW);
             if (S == 0 || (pairs && H->lz_tma)) continue;
             int stages = bzk::kLzMaxStages;
-            while (stages >= 3 && bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end > (size_t)H->smem_optin) --stages;
-            if (stages < 3) continue;
+            while (stages >= bzk::kLzMinStages && bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end > (size_t)H->smem_optin) --stages;
+            if (stages < bzk::kLzMinStages) continue;
             const size_t smem = bzk::lz_offsets(nvt, mcap, G, stages, S, VW).end;
             int occ = 0;
             const bzk::LzKernel kern = lz_kernel(H, G, ST);

@@ -59,7 +59,8 @@ __host__ __device__ constexpr int lz_threads(int ST) { return ST + kLzCollT; }
 constexpr int kLzDParts = 8;       // slots of the increment sums per cell
 constexpr int kLzMaxG = 4;         // cells per CTA group
 constexpr int kLzMaxN = 32;        // velocity nodes per axis (N^2 / 4 <= 256)
-constexpr int kLzMaxStages = 5;    // streaming stages staged per thread (at least 2)
+constexpr int kLzMaxStages = 5;    // streaming stages staged per thread (at least kLzMinStages)
+constexpr int kLzMinStages = 3;    // (two: 256^2 x 32^3 6.28 -> 6.76 ms)
 constexpr unsigned long long kLzWaitNs = 1000000000ull;   // an mbarrier wait gives up after 1 s
 
 // meta layout: [0] M, [1] overflow (M > mcap), [2] E (terms of the step),
@@ -920,14 +921,6 @@ __device__ __forceinline__ void lz_mono_from_powers(const float (&s)[5], float y
     M[25] += yz * t2;
 }
 
-// The same sums for one node value d at velocity (x, y, z).
-__device__ __forceinline__ void lz_mono_node(float d, float x, float y, float z, float (&M)[32])
-{
-    const float x2 = x * x;
-    const float s[5] = {d, d * x, d * x2, d * x2 * x, d * x2 * x2};
-    lz_mono_from_powers(s, y, z, M);
-}
-
 // Sum of 32 values over a warp, left with lane l holding the total of value l
 // (recursive halving: 31 shuffles instead of 32 x 5).
 __device__ __forceinline__ float lz_warp_reduce_scatter(float (&v)[32])
@@ -1480,19 +1473,20 @@ __device__ __forceinline__ void lz_terms_done_wait()
 }
 constexpr int kLzTailChunk = 256;  // active nodes per claimed chunk of the increment sums
 
-// One CTA of 512 threads per SM, two roles working on consecutive groups of
-// G cells: warps 0-7 stream group i (Eq. streaming2D, the power sums, the
-// active nodes to one compact array) and then solve the correction and the
-// moments of group i - 2, while warps 8-15 apply the collision terms, their
-// sums and the write-back of group i - 1 from the other compact array.
-// Streaming is bound by HBM and the collision terms by shared memory, so
-// the two overlap.
+// One CTA per SM, two roles working on consecutive groups of G cells: the first
+// ST / 32 warps stream group i (Eq. streaming2D, the power sums, the active nodes
+// to one compact array), while the last eight solve the correction and the
+// moments of group i - 2 (a warp per cell) and then apply the collision terms,
+// their sums and the write-back of group i - 1 from the other compact array.
+// Streaming is bound by HBM and its instructions and the collision terms by
+// shared memory, so the two overlap.
 //
 // NV: the velocity axis length as a compile-time constant (0: read g.nv at
 // run time).  SX: stretched cells (per-column and per-row Courant factors
 // g.sx, g.sy).  Streaming thread t < S = K N^2/4 owns node quad q = t mod
 // (N^2/4) (four consecutive jz at one (jx, jy)) of jx-plane t div (N^2/4) of
-// every stage; a stage covers K planes and a cell J = N / K stages.
+// every stage; a stage covers K planes and a cell J = N / K stages.  VW = 2: node
+// pairs in place of quads, N^2/2 of them to a plane.
 //
 // TMA: the streaming sources arrive by bulk copies (cp.async.bulk) that
 // thread 0 of the role issues into a ring of slots, with a full
@@ -1768,9 +1762,9 @@ __device__ __forceinline__ void lz_run(const Geo &g, const LzArgs &a, char *smem
                 }
             }
             if (clk && t == 0) a.clk[it * kClkPhases + 1] = clock64();
-            if (clk && t == 0) a.clk[it * kClkPhases + 5] = clock64();
         } else {
             solve(it, warp - kStreamWarps);
+            if (clk && t == ST) a.clk[it * kClkPhases + 5] = clock64();
         }
         if (!streamer && it >= 1 && it <= nmine) {
             const int tc = t - ST, buf = (it - 1) & 1;
