@@ -373,13 +373,16 @@ __device__ __forceinline__ void rx_run(int n, const uint32_t *__restrict__ list,
 
 // Threads of a CTA for a shared set: those of the columns, and in FP32 (64 registers a
 // thread) as many more as its share of an SM has room for, which help with the samples
-// and the sorted terms: 24^3 with 10^4 samples 767 -> 632 us for 64^2 cells (with rx_run), with
-// 500 samples 412 -> 450, so only from a quarter as many samples as nodes.
+// and the sorted terms, from 0.3 times as many samples as nodes.  64^2 cells, us with the
+// columns' threads / with more, at 0.1, 0.25, 0.35 and 0.8 samples per node: 24^3
+// 468 / 477, 517 / 521, 558 / 545, 714 / 664; 20^3 264 / 265, 291 / 291, 310 / 308, 391 /
+// 378; 21^3 286 / 289, 317 / 319, 335 / 338, 418 / 418; up to 16^3 the CTAs that share
+// an SM leave no room for more.
 template <typename R>
 inline int rx_threads(int N, int nvt, int nseg, int nt, size_t smem_sm)
 {
     const int T = (N * N * nseg + 31) / 32 * 32;
-    if (sizeof(R) == 8 || nt < nvt / 4) return T;
+    if (sizeof(R) == 8 || 10 * nt < 3 * nvt) return T;
     const size_t need = rx_smem<R>(nullptr, nullptr, N, nvt, kMaxThreads, nt) + 1024;
     const int ctas = (int)(smem_sm / need);
     return ctas < 1 ? T : std::max(T, kMaxThreads / ctas / 32 * 32);
