@@ -90,10 +90,11 @@ bz_status scratch_address(int dev, unsigned char **out)
 }
 
 // The cells with separate increments (bz_relax.cuh) where their two slabs and
-// products fit a block's shared memory and the destination-sorted terms fit
-// the scratch array (up to about 36000 FP64 or 48000 FP32 samples): no
-// shared-memory atomics.  64^2 x 24^3 FP32, 10^4 samples: 1052
-// -> 630 us a call.
+// products fit a block's shared memory (227 KB: at 24^3 in FP32 up to about 29000
+// samples, at 12^3 in FP64 about 24000), which is the limit, and the
+// destination-sorted terms the scratch array (2 MiB for 32 bytes a sample in FP32
+// or 40 in FP64, and 8 a node: it never is): no shared-memory atomics.  64^2 x 24^3
+// FP32, 10^4 samples: 1052 -> 630 us a call.
 // Returns false (nothing launched) otherwise; *e is the launches' status.
 template <typename R>
 bool run_relax(const bzk::Geo &g, unsigned char *scr, const int64_t *stepp, int64_t step, const void *hin, void *hout,
