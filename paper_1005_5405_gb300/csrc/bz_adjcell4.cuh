@@ -22,8 +22,8 @@
 // A thread owns quads of four jz nodes of one jy row in J consecutive jx-planes
 // (quads of a row are rotated by jx so that gathers spread over the banks).
 //
-// Bound: latency between ten barriers and the shared-memory gathers (about 17
-// thousand wavefronts of a cell's 28 thousand cycles at 20^3 with 5000 samples,
+// Bound: latency between ten barriers and the shared-memory gathers (17.0
+// thousand wavefronts of a cell's 30 thousand cycles at 20^3 with 5000 samples,
 // two CTAs of 512 threads an SM); HBM needs only 0.5 of its 1.8 ms a step at
 // 128^2.  Against the forward kernel's body with a transposed tail (gathers twice
 // per loss term, three reductions, two solves by one lane after another, sums
