@@ -112,7 +112,7 @@ def kernel_source_hash(files):
 
 # The per-cell kernel a handle runs (bz_info.kernel_variant), the ncu summary
 # of its 64x64-cell profiling case, and the headers its device code lives in.
-CELL_KERNELS = {0: ("k_cell<fused>", None, ()),
+CELL_KERNELS = {0: ("k_relax (k_cell where two slabs do not fit)", None, ()),
                 1: ("k_cell4<fused>", "k_cell_fused_cavity64_v32.md",
                     ("bz_kernels.cuh", "bz_cell4.cuh")),
                 2: ("k_lz", "k_lz_cavity64_v32.md",
